@@ -108,9 +108,23 @@ __device__ __forceinline__ void store_or_fold(const EvalArgs &a, double (&acc)[9
         const int p = ibase + (e - q * itile);
         if (p >= a.n_act)
             continue;
+        // eight partials in flight at a time (each load is an L2 round trip),
+        // added in index order
+        const double *pp = &a.part[static_cast<size_t>(q) * a.n_act + p];
+        const size_t step = static_cast<size_t>(9) * a.n_act;
         double s = 0.0;
-        for (int sp = 0; sp < a.split; ++sp)
-            s += __ldcg(&a.part[(static_cast<size_t>(sp) * 9 + q) * a.n_act + p]);
+        int sp = 0;
+        for (; sp + 8 <= a.split; sp += 8) {
+            double v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                v[u] = __ldcg(pp + (sp + u) * step);
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                s += v[u];
+        }
+        for (; sp < a.split; ++sp)
+            s += __ldcg(pp + sp * step);
         a.out[static_cast<size_t>(q) * a.ostride + p] = s;
     }
     if (threadIdx.x == 0)
@@ -601,96 +615,101 @@ cudaError_t nb_eval_smem_setup()
     return cudaSuccess;
 }
 
-// Blocks of the chosen evaluation kernel that fit on one SM.
-int resident_blocks(const nb_ctx *c, const nb_tiles &t)
+// Relative cost of a pair term by the number of lanes that share an i: lane
+// l reads its own j records, so the shared-memory reads of a warp spread over
+// lanes x 16 bytes per row (one i per lane: a broadcast).  Measured on GB300
+// with the chip full (2^20 j, 1024 active; EX and FP64 8192 j).
+double lane_cost(bool mixed, bool ex, int lanes)
 {
-    const bool mixed = nb_fp32_eval(c->cfg.precision);
-    const bool ex = c->cfg.precision == NB_EX;
-    const size_t smem = static_cast<size_t>(2) * (ex ? kRecBytesEx : mixed ? kRecBytes32 : kRecBytes64) * t.jtile +
-                        (mixed ? static_cast<size_t>(18) * t.ki * t.threads * sizeof(float) : 0) +
-                        (!mixed && !ex && fp64_shared_totals(t.ki)
-                             ? static_cast<size_t>(9) * t.ki * t.threads * sizeof(double) : 0);
-    int nb = 0;
-    cudaError_t e;
-    if (ex) {
-        if (t.junroll == 1) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eval_ex_kernel<float>, t.threads, smem);
-        else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eval_ex_kernel<float2>, t.threads, smem);
-    } else if (mixed) {
-        const EvalKernel k = mixed_kernel(t.ki, t.junroll, t.jtile);
-        e = k ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, t.threads, smem) : cudaErrorInvalidValue;
-    } else {
-        if (t.ki == 1) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eval_fp64_kernel<1>, t.threads, smem);
-        else if (t.ki == 2) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eval_fp64_kernel<2>, t.threads, smem);
-        else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eval_fp64_kernel<4>, t.threads, smem);
-    }
-    if (e != cudaSuccess || nb < 1) {
-        (void)cudaGetLastError();
-        return 1;
-    }
-    return nb;
+    constexpr double kMixed[6] = {1.0, 1.0, 1.06, 1.15, 1.33, 1.65};
+    constexpr double kEx[6] = {1.0, 1.0, 1.0, 1.06, 1.3, 1.5};
+    constexpr double kFp64[6] = {1.0, 1.0, 1.0, 1.02, 1.04, 1.06};
+    int k = 0;
+    while ((1 << k) < lanes)
+        ++k;
+    return mixed ? kMixed[k] : ex ? kEx[k] : kFp64[k];
 }
 
-// Automatic launch shape.  Large active sets: one i per thread slot, no
-// split.  Small ones: lanes share an i so that a block's i-slots are not
-// mostly empty, and the j-range is split across blocks until the grid
-// covers every SM several times.
+// Automatic launch shape: the (ki, lanes, split) with the smallest estimated
+// time.  A block holds itile = threads / lanes * ki i-slots (idle ones cost
+// as much as used ones, so a ragged active set wants small i-tiles) and one
+// of `split` j-chunks; G = i-tiles x split blocks give an SM k = ceil(G / SMs)
+// of them to work through, at the kernel's full rate once enough warps are
+// resident (two 128-thread blocks in the FP32 kernels, one in FP64, whose
+// pipe one warp per scheduler fills); more, smaller blocks even out (6 % / k:
+// 1024 of 2^20 mixed, k = 2 1982 us, k = 6 1934).  To that come a launch's
+// fixed part per wave and the last block's fold of the split partial sums.  Lanes take over
+// from the split where the active set is small: they need no fold.  Before, the
+// split could not go below two whole j-tiles, which left small systems on a few
+// SMs: 1024 particles FP64 950 us (16 blocks), now 116; EX 309 -> 32; mixed
+// 51 -> 18; 130 of 65537 mixed 127 -> 45; 384 of 8192 EX 319 -> 69.  Over a
+// sweep of 19 sizes the choice is within 3 % or 3 us of the best shape, and
+// 16 % at the worst (130 of 65537 mixed: lanes 16, split 36 39 us).
 nb_tiles nb_auto_tiles(const nb_ctx *c, int64_t n_act, const nb_tiles &req, int64_t j_count)
 {
-    nb_tiles t = req;
     const bool ex = c->cfg.precision == NB_EX;
     const bool mixed = nb_fp32_eval(c->cfg.precision);
-    // defaults from the launch-shape sweeps on GB300 (autotune.py): mixed
-    // KI = 2 with four j per iteration for small active sets, three
-    // i-particles per thread and 512-j tiles from 8192 active on
-    const bool big = n_act >= 8192;
-    if (t.ki <= 0)
-        t.ki = mixed ? (big ? 3 : 2) : 1;
-    if (t.threads <= 0)
-        t.threads = ex ? kExThreads : mixed ? mixed_max_threads(t.ki) : 128;
-    if (t.junroll <= 0)
-        t.junroll = ex ? 2 : 4;
-    if (t.lanes <= 0) {
-        // two lanes per i-particle below 4096 active in the mixed kernel
-        // (fewer, deeper j-chunks to fold); more while the block would hold
-        // more i-slots than there are active particles
-        int l = mixed && t.ki == 2 && n_act < 4096 ? 2 : 1;
-        while (l < 32 && static_cast<int64_t>(t.threads / (2 * l)) * t.ki >= n_act)
-            l *= 2;
-        t.lanes = l;
-    }
-    if (t.jtile <= 0)
-        t.jtile = mixed ? (n_act >= 512 ? 512 : 256) : (ex ? 512 : 256);
-    if ((mixed || ex) && t.jtile % 4)
-        t.jtile = (t.jtile / 4 + 1) * 4;   // whole 16-byte rows per bulk copy
-    if (t.split <= 0) {
-        // Split the j-range so that the grid fills whole waves of resident
-        // blocks: all blocks of a launch do equal work, so a partial last
-        // wave idles the rest of the GPU for a whole block's duration.
-        const int64_t jn = j_count > 0 ? j_count : ((mixed || ex) ? c->npad : c->n);
-        const int64_t itile = static_cast<int64_t>(t.threads / t.lanes) * t.ki;
-        const int64_t nblk = (n_act + itile - 1) / itile;
-        const int64_t cap = static_cast<int64_t>(c->sm_count) * resident_blocks(c, t);
-        const int64_t max_s = std::max<int64_t>(1, std::min<int64_t>(1024, jn / (2 * t.jtile)));
-        // Each block does 1/s of an i-tile's work, so the launch takes about
-        // ceil(nblk s / cap) / s block-times; take the smallest s within 2 %
-        // of the best (fewer partial sums to fold).
-        int64_t best = 1;
-        if (nblk < 4 * cap) {
-            double tmin = 1e300;
-            std::vector<double> ts(static_cast<size_t>(max_s) + 1, 0.0);
-            for (int64_t s = 1; s <= max_s; ++s) {
-                ts[s] = static_cast<double>((nblk * s + cap - 1) / cap) / static_cast<double>(s);
-                tmin = std::min(tmin, ts[s]);
-            }
-            for (int64_t s = 1; s <= max_s; ++s)
-                if (ts[s] <= 1.02 * tmin) {
-                    best = s;
+    const int64_t sms = c->sm_count;
+    const int64_t jn = j_count > 0 ? j_count : ((mixed || ex) ? c->npad : c->n);
+    const int64_t na = std::max<int64_t>(1, n_act);
+    // pairs per microsecond and SM with the chip full
+    constexpr double kMixedRate[4] = {0.0, 3650.0, 3780.0, 3950.0};
+    constexpr double kExRate = 454.0, kFp64Rate = 69.7;
+
+    auto jtile_for = [&](int ki, int64_t chunk) {
+        if (req.jtile > 0)
+            return (mixed || ex) ? (req.jtile + 3) / 4 * 4 : req.jtile;  // whole 16-byte rows per bulk copy
+        const bool wide = chunk >= 512 && (ex || (mixed && ki > 1));
+        return wide ? 512 : 256;
+    };
+    // a partly given shape keeps a fixed ki, so that which requests fit does
+    // not depend on the estimate
+    const bool given = req.ki > 0 || req.threads > 0 || req.jtile > 0 || req.junroll > 0;
+    const int ki_lo = req.ki > 0 ? req.ki : !mixed ? 1 : !given ? 1 : n_act >= 8192 ? 3 : 2;
+    const int ki_hi = mixed && !given ? 3 : ki_lo;
+    nb_tiles best{};
+    double tbest = 1e300;
+    for (int ki = ki_lo; ki <= ki_hi; ++ki) {
+        const int threads = req.threads > 0 ? req.threads
+                            : ex            ? kExThreads
+                            : mixed         ? (given ? mixed_max_threads(ki) : 128)
+                                            : 128;
+        const int ju = req.junroll > 0 ? req.junroll : ex ? 2 : 4;
+        const double rate = mixed ? kMixedRate[std::min(ki, 3)] : ex ? kExRate : kFp64Rate;
+        const double fill = (mixed || ex) ? 256.0 : 128.0;  // threads that reach the full rate
+        for (int lanes = req.lanes > 0 ? req.lanes : 1; lanes <= (req.lanes > 0 ? req.lanes : 32); lanes *= 2) {
+            const int64_t itile = static_cast<int64_t>(std::max(1, threads / lanes)) * ki;
+            const int64_t nblk = (na + itile - 1) / itile;
+            const int64_t grain = std::max<int64_t>((mixed || ex) ? 4 : 1, (mixed || ex) ? lanes * ju : lanes);
+            for (const int w : {1, 2, 3, 4, 6, 8, 12, 16}) {
+                int64_t split = req.split > 0 ? req.split : std::max<int64_t>(1, sms * w / nblk);
+                if (req.split <= 0 && split > 1024)
                     break;
+                int64_t chunk = (jn + split - 1) / split;
+                chunk = std::max<int64_t>(grain, (chunk + grain - 1) / grain * grain);
+                if (req.split <= 0)
+                    split = (jn + chunk - 1) / chunk;
+                const int64_t k = (nblk * split + sms - 1) / sms;
+                double t = static_cast<double>(chunk * itile) * lane_cost(mixed, ex, lanes) / rate *
+                           std::max(static_cast<double>(k), fill / threads) * (1.0 + 0.06 / static_cast<double>(k));
+                t += static_cast<double>((k + 1) / 2) * (mixed ? 2.0 * ki : ex ? 2.5 : 4.0);
+                if (split > 1)
+                    t += 1.0 + static_cast<double>((9 * itile + threads - 1) / threads * split) / 16.0;
+                if (t < tbest) {
+                    tbest = t;
+                    best.ki = ki;
+                    best.threads = threads;
+                    best.lanes = lanes;
+                    best.split = static_cast<int32_t>(split);
+                    best.junroll = ju;
+                    best.jtile = jtile_for(ki, chunk);
                 }
+                if (req.split > 0)
+                    break;
+            }
         }
-        t.split = static_cast<int32_t>(best);
     }
-    return t;
+    return best;
 }
 
 cudaError_t nb_launch_eval(nb_ctx *c, const EvalLaunch &L)
@@ -719,14 +738,15 @@ cudaError_t nb_launch_eval(nb_ctx *c, const EvalLaunch &L)
     const int itile = (t.threads / t.lanes) * t.ki;
     const int gx = (L.n_act + itile - 1) / itile;
     // j-range (the whole buffer unless L.j1 >= 0) and chunk per split, a
-    // whole number of tiles
+    // whole number of the lanes' inner iterations (and of 16-byte rows)
     const int64_t nbuf = (mixed || ex) ? c->npad : c->n;
     const int64_t j0 = L.j1 >= 0 ? L.j0 : 0, j1 = L.j1 >= 0 ? L.j1 : nbuf;
     if (j0 < 0 || j1 > nbuf || j0 > j1 || ((mixed || ex) && (j0 % 4 || j1 % 4)))
         return cudaErrorInvalidValue;
     const int64_t jn = j1 - j0;
     int64_t chunk = std::max<int64_t>(1, (jn + t.split - 1) / t.split);
-    chunk = (chunk + t.jtile - 1) / t.jtile * t.jtile;
+    const int64_t grain = std::max(mixed || ex ? 4 : 1, t.lanes * (mixed || ex ? t.junroll : 1));
+    chunk = (chunk + grain - 1) / grain * grain;
     const int split = std::max(1, static_cast<int>((jn + chunk - 1) / chunk));
 
     EvalArgs a;
