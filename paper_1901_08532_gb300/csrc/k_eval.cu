@@ -645,7 +645,7 @@ double lane_cost(bool mixed, bool ex, int lanes)
 // 51 -> 18; 130 of 65537 mixed 127 -> 45; 384 of 8192 EX 319 -> 69.  Over a
 // sweep of 19 sizes the choice is within 3 % or 3 us of the best shape, and
 // 16 % at the worst (130 of 65537 mixed: lanes 16, split 36 39 us).
-nb_tiles nb_auto_tiles(const nb_ctx *c, int64_t n_act, const nb_tiles &req, int64_t j_count)
+nb_tiles nb_auto_tiles(const nb_ctx *c, int64_t n_act, const nb_tiles &req, int64_t j_count, double *us)
 {
     const bool ex = c->cfg.precision == NB_EX;
     const bool mixed = nb_fp32_eval(c->cfg.precision);
@@ -709,7 +709,52 @@ nb_tiles nb_auto_tiles(const nb_ctx *c, int64_t n_act, const nb_tiles &req, int6
             }
         }
     }
+    if (us)
+        *us = tbest;
     return best;
+}
+
+// Partial sums and arrival counters of a j-split launch, grown on demand.
+// Outgrown blocks stay allocated until nb_free (a captured graph may hold
+// them); doubling bounds them by the size of the last.  False where the memory
+// cannot be allocated now.
+static bool ensure_split_scratch(nb_ctx *c, size_t doubles, int tiles)
+{
+    const bool grow_part = doubles > c->part_cap, grow_cnt = static_cast<size_t>(tiles) > c->tile_cnt_cap;
+    if (!grow_part && !grow_cnt)
+        return true;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    if (grow_part) {
+        const size_t cap_new = std::max(doubles, 2 * c->part_cap);
+        void *p = nullptr;
+        if (cudaMalloc(&p, cap_new * sizeof(double)) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return false;
+        }
+        if (c->part)
+            c->outgrown.push_back(c->part);
+        c->part = static_cast<double *>(p);
+        c->part_cap = cap_new;
+    }
+    if (grow_cnt) {
+        const size_t cap_new = std::max(static_cast<size_t>(tiles), 2 * c->tile_cnt_cap);
+        void *p = nullptr;
+        if (cudaMalloc(&p, cap_new * sizeof(unsigned)) != cudaSuccess ||
+            cudaMemsetAsync(p, 0, cap_new * sizeof(unsigned), c->stream) != cudaSuccess) {
+            cudaFree(p);
+            (void)cudaGetLastError();
+            return false;
+        }
+        if (c->tile_cnt)
+            c->outgrown.push_back(c->tile_cnt);
+        c->tile_cnt = static_cast<unsigned *>(p);
+        c->tile_cnt_cap = cap_new;
+    }
+    return true;
 }
 
 cudaError_t nb_launch_eval(nb_ctx *c, const EvalLaunch &L)
@@ -747,7 +792,7 @@ cudaError_t nb_launch_eval(nb_ctx *c, const EvalLaunch &L)
     int64_t chunk = std::max<int64_t>(1, (jn + t.split - 1) / t.split);
     const int64_t grain = std::max(mixed || ex ? 4 : 1, t.lanes * (mixed || ex ? t.junroll : 1));
     chunk = (chunk + grain - 1) / grain * grain;
-    const int split = std::max(1, static_cast<int>((jn + chunk - 1) / chunk));
+    int split = std::max(1, static_cast<int>((jn + chunk - 1) / chunk));
 
     EvalArgs a;
     a.jb = (mixed || ex) ? static_cast<const void *>(c->jf32) : static_cast<const void *>(c->jb64);
@@ -768,29 +813,14 @@ cudaError_t nb_launch_eval(nb_ctx *c, const EvalLaunch &L)
     a.cnt = nullptr;
     a.tx_extra = c->inject == 1 ? 16u : 0u;
     c->inject = 0;
+    if (split > 1 && !ensure_split_scratch(c, static_cast<size_t>(split) * 9 * L.n_act, gx)) {
+        // no scratch to be had (the stream is being captured, or no memory):
+        // one block per i-tile takes the whole j-range
+        split = 1;
+        a.split = 1;
+        a.jchunk = static_cast<int>((jn + grain - 1) / grain * grain);
+    }
     if (split > 1) {
-        const size_t need = static_cast<size_t>(split) * 9 * L.n_act;
-        if (need > c->part_cap) {
-            cudaFree(c->part);
-            c->part = nullptr;
-            c->part_cap = 0;
-            cudaError_t e = cudaMalloc(&c->part, need * sizeof(double));
-            if (e != cudaSuccess)
-                return e;
-            c->part_cap = need;
-        }
-        if (static_cast<size_t>(gx) > c->tile_cnt_cap) {
-            cudaFree(c->tile_cnt);
-            c->tile_cnt = nullptr;
-            c->tile_cnt_cap = 0;
-            cudaError_t e = cudaMalloc(&c->tile_cnt, static_cast<size_t>(gx) * sizeof(unsigned));
-            if (e != cudaSuccess)
-                return e;
-            e = cudaMemsetAsync(c->tile_cnt, 0, static_cast<size_t>(gx) * sizeof(unsigned), c->stream);
-            if (e != cudaSuccess)
-                return e;
-            c->tile_cnt_cap = gx;
-        }
         a.part = c->part;
         a.cnt = c->tile_cnt;
     }

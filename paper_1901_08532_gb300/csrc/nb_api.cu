@@ -116,8 +116,36 @@ nb_status sync_ctl(nb_ctx *c)
     return NB_OK;
 }
 
-nb_status eval_on_device(nb_ctx *c, const int32_t *act_dev, int64_t n_act)
+// The complete active set 0 .. n-1 against all particles, each unordered pair
+// once (k_sym.cu), where the context's plan for it is estimated faster than the
+// ordinary kernels and no launch shape is asked for.  *done says whether it
+// ran.
+nb_status eval_all_pairs(nb_ctx *c, double *out, bool *done)
 {
+    *done = false;
+    const nb_tiles &t = c->cfg.tiles;
+    if (!c->sym_use || c->inject || t.ki || t.threads || t.jtile || t.lanes || t.split || t.junroll)
+        return NB_OK;
+    const bool rows = nb_jrows(c->cfg.precision) > 0;
+    int launches = 0;
+    CU(c, nb_launch_sym(c->cfg.precision, c->sym_plan, rows ? static_cast<const void *>(c->jf32) : c->jb64,
+                        static_cast<size_t>(rows ? c->npad : c->n), static_cast<int>(c->n), c->eps * c->eps,
+                        c->sym_work, out, static_cast<size_t>(c->n), c->stream, &launches));
+    c->launches += launches;
+    c->interactions += static_cast<double>(c->n) * static_cast<double>(c->n);
+    *done = true;
+    return NB_OK;
+}
+
+// all: the list is 0 .. n-1.
+nb_status eval_on_device(nb_ctx *c, const int32_t *act_dev, int64_t n_act, bool all)
+{
+    if (all) {
+        bool done;
+        const nb_status s = eval_all_pairs(c, c->anew, &done);
+        if (s != NB_OK || done)
+            return s;
+    }
     EvalLaunch L;
     L.act = act_dev;
     L.n_act = static_cast<int>(n_act);
@@ -137,7 +165,7 @@ nb_status advance(nb_ctx *c, double tn, int64_t n_act)
 {
     std::swap(c->act, c->act_next);
     CU(c, nb_launch_predict(c, tn));
-    nb_status s = eval_on_device(c, c->act, n_act);
+    nb_status s = eval_on_device(c, c->act, n_act, n_act == c->n);  // ascending: all of them
     if (s != NB_OK)
         return s;
     CU(c, nb_launch_correct(c, tn, static_cast<int>(n_act)));
@@ -272,6 +300,9 @@ void free_all(nb_ctx *c)
     cudaFree(c->stage);
     cudaFree(c->part);
     cudaFree(c->tile_cnt);
+    cudaFree(c->sym_work);
+    for (void *p : c->outgrown)
+        cudaFree(p);
     cudaFree(c->blk);
     cudaFree(c->red);
     cudaFree(c->ctl);
@@ -388,12 +419,26 @@ nb_status nb_init(nb_ctx **out, int64_t n, const double *m, const double *x, con
     CUI(cudaGetDevice(&c->dev));
     CUI(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->dev));
     CUI(nb_eval_smem_setup());
+    CUI(nb_sym_smem_setup());
     const size_t N = static_cast<size_t>(n);
     CUI(cudaMalloc(&c->m, N * sizeof(double)));
     CUI(cudaMalloc(&c->st, 18 * N * sizeof(double)));
     CUI(cudaMalloc(&c->t, N * sizeof(double)));
     CUI(cudaMalloc(&c->dt, N * sizeof(double)));
     c->npad = (n + 3) / 4 * 4;
+    {
+        double us = 0.0;
+        (void)nb_auto_tiles(c, n, nb_tiles{}, 0, &us);
+        c->sym_plan = nb_sym_plan(cf.precision, n, c->sm_count);
+        c->sym_use = c->sym_plan.us < us;
+        // its workspace, so that no evaluation allocates; without the memory
+        // the ordinary kernels run
+        if (c->sym_use && cudaMalloc(&c->sym_work, c->sym_plan.bytes) != cudaSuccess) {
+            (void)cudaGetLastError();
+            c->sym_work = nullptr;
+            c->sym_use = false;
+        }
+    }
     if (const int rows = nb_jrows(cf.precision)) {
         CUI(cudaMalloc(&c->jf32, rows * static_cast<size_t>(c->npad) * sizeof(float)));
         CUI(cudaMemsetAsync(c->jf32, 0, rows * static_cast<size_t>(c->npad) * sizeof(float), c->stream));
@@ -434,7 +479,7 @@ nb_status nb_init(nb_ctx **out, int64_t n, const double *m, const double *x, con
     }
     for (int pass = 0; pass < 2; ++pass) {
         CUI(nb_launch_predict(c, 0.0));
-        nb_status s = eval_on_device(c, c->act, n);
+        nb_status s = eval_on_device(c, c->act, n, true);
         if (s != NB_OK)
             return bail(s);
         CUI(nb_launch_init_state(c, pass));
@@ -517,10 +562,15 @@ nb_status nb_evaluate(nb_ctx *c, const int32_t *active, int64_t n_act, int activ
         return fail(c, NB_EINVAL, "n_act must be in [0, n]");
     if (!active && n_act != c->n)
         return fail(c, NB_EINVAL, "active == NULL requires n_act == n");
+    bool all = n_act == c->n;  // the list is 0 .. n-1 (a device list is not looked at)
     if (active && !active_on_device)
-        for (int64_t k = 0; k < n_act; ++k)
+        for (int64_t k = 0; k < n_act; ++k) {
             if (active[k] < 0 || active[k] >= c->n)
                 return fail(c, NB_EINVAL, "active index out of range");
+            all = all && active[k] == k;
+        }
+    else if (active)
+        all = false;
     if (n_act > 0) {
         if (!active)
             CU(c, nb_launch_iota(c, static_cast<int>(c->n), c->act));
@@ -528,7 +578,7 @@ nb_status nb_evaluate(nb_ctx *c, const int32_t *active, int64_t n_act, int activ
             CU(c, cudaMemcpyAsync(c->act, active, static_cast<size_t>(n_act) * sizeof(int32_t),
                                   active_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                                   c->stream));
-        nb_status s = eval_on_device(c, c->act, n_act);
+        nb_status s = eval_on_device(c, c->act, n_act, all);
         if (s != NB_OK)
             return s;
     }
@@ -573,17 +623,25 @@ nb_status nb_schedule(nb_ctx *c, double *t_next, int64_t *n_act)
     return NB_OK;
 }
 
-// Copy an active list into c->act (checked when it is a host list).
-nb_status load_active(nb_ctx *c, const int32_t *active, int64_t n_act, int active_on_device)
+// Copy an active list into c->act (checked when it is a host list); *all: it
+// is 0 .. n-1 (a device list is not looked at).
+nb_status load_active(nb_ctx *c, const int32_t *active, int64_t n_act, int active_on_device, bool *all = nullptr)
 {
     if (n_act < 0 || n_act > c->n)
         return fail(c, NB_EINVAL, "n_act must be in [0, n]");
     if (!active && n_act != c->n)
         return fail(c, NB_EINVAL, "active == NULL requires n_act == n");
+    bool identity = n_act == c->n;
     if (active && !active_on_device)
-        for (int64_t k = 0; k < n_act; ++k)
+        for (int64_t k = 0; k < n_act; ++k) {
             if (active[k] < 0 || active[k] >= c->n)
                 return fail(c, NB_EINVAL, "active index out of range");
+            identity = identity && active[k] == k;
+        }
+    else if (active)
+        identity = false;
+    if (all)
+        *all = identity;
     if (n_act == 0)
         return NB_OK;
     if (!active)
@@ -608,13 +666,20 @@ nb_status nb_evaluate_partial(nb_ctx *c, const int32_t *active, int64_t n_act, i
         return fail(c, NB_EINVAL, "j-range must satisfy 0 <= j_lo <= j_hi <= n");
     if (rows && (j_lo % 4 || (j_hi % 4 && j_hi != c->n)))
         return fail(c, NB_EINVAL, "FP32-row precisions need j_lo and j_hi multiples of 4 (or j_hi == n)");
-    nb_status s = load_active(c, active, n_act, active_on_device);
+    bool all = false;
+    nb_status s = load_active(c, active, n_act, active_on_device, &all);
     if (s != NB_OK)
         return s;
     // the partial sums overwrite the context's evaluation results
     c->have_eval = false;
     if (n_act == 0)
         return NB_OK;
+    bool done = false;
+    if (all && j_lo == 0 && j_hi == c->n) {  // as in nb_step, to the bit
+        s = eval_all_pairs(c, part_on_device ? part : c->anew, &done);
+        if (s != NB_OK)
+            return s;
+    }
     EvalLaunch L;
     L.act = c->act;
     L.n_act = static_cast<int>(n_act);
@@ -622,11 +687,13 @@ nb_status nb_evaluate_partial(nb_ctx *c, const int32_t *active, int64_t n_act, i
     L.out = part_on_device ? part : c->anew;
     L.j0 = j_lo;
     L.j1 = rows && j_hi == c->n ? c->npad : j_hi;
-    L.tiles = nb_auto_tiles(c, n_act, c->cfg.tiles, L.j1 - L.j0);
-    cudaError_t e = nb_launch_eval(c, L);
-    if (e == cudaErrorInvalidValue)
-        return fail(c, NB_EINVAL, "evaluation launch shape is not valid for this size");
-    CU(c, e);
+    if (!done) {
+        L.tiles = nb_auto_tiles(c, n_act, c->cfg.tiles, L.j1 - L.j0);
+        cudaError_t e = nb_launch_eval(c, L);
+        if (e == cudaErrorInvalidValue)
+            return fail(c, NB_EINVAL, "evaluation launch shape is not valid for this size");
+        CU(c, e);
+    }
     if (!part_on_device) {
         CU(c, cudaMemcpyAsync(part, c->anew, static_cast<size_t>(9 * n_act) * sizeof(double),
                               cudaMemcpyDeviceToHost, c->stream));

@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <vector>
 
 #include "nb.h"
 
@@ -41,6 +42,19 @@ struct nb_ctl {                      // small device control block
 #define NB_ERR_NONFINITE 1
 #define NB_ERR_TIMEOUT 2
 
+// Evaluation of a complete active set with each unordered pair once (k_sym.cu).
+// Launch plan for n particles: the kernel (kind), T tiles, k offsets per block, j-tiles in
+// `parts`, nd offsets per launch, row length ns and number of the i-slots,
+// workspace bytes, estimated time.
+struct SymPlan {
+    double us = 1e300;
+    int kind = 0, T = 0, k = 1, parts = 1, nd = 1;
+    size_t ns = 0, pi_slots = 0, bytes = 0;
+};
+// Bytes of partial sums that a plan may use where it needs more than the two
+// slots (72 B per particle each) of the smallest one.
+constexpr double kSymSlotBytes = 1e9;
+
 struct nb_ctx {
     int dev = 0;
     cudaStream_t stream = nullptr;
@@ -64,6 +78,10 @@ struct nb_ctx {
     size_t part_cap = 0;       // doubles
     unsigned *tile_cnt = nullptr;
     size_t tile_cnt_cap = 0;
+    std::vector<void *> outgrown;  // earlier, smaller blocks of part and tile_cnt
+    SymPlan sym_plan;          // evaluation of all particles, each pair once
+    bool sym_use = false;
+    void *sym_work = nullptr;  // its partial sums
     int32_t *blk = nullptr;    // scheduler block counts
     double *red = nullptr;     // reduction scratch
     size_t red_cap = 0;        // doubles
@@ -217,8 +235,17 @@ struct EvalLaunch {
 // k_eval.cu
 cudaError_t nb_launch_eval(nb_ctx *c, const EvalLaunch &L);
 // j_count: length of the j-range evaluated (0: the whole buffer)
-nb_tiles nb_auto_tiles(const nb_ctx *c, int64_t n_act, const nb_tiles &req, int64_t j_count = 0);
+// *us: the estimated time
+nb_tiles nb_auto_tiles(const nb_ctx *c, int64_t n_act, const nb_tiles &req, int64_t j_count = 0,
+                       double *us = nullptr);
 cudaError_t nb_eval_smem_setup();
+// k_sym.cu
+SymPlan nb_sym_plan(int precision, int64_t n, int sms);
+cudaError_t nb_sym_smem_setup();
+// jb, np: predicted particles and row stride; work: plan.bytes of device
+// memory, 256-byte aligned; out [9][ostride]; *launches counts kernels.
+cudaError_t nb_launch_sym(int precision, const SymPlan &plan, const void *jb, size_t np, int n, double eps2,
+                          void *work, double *out, size_t ostride, cudaStream_t stream, int *launches);
 // k_predict.cu
 cudaError_t nb_launch_predict(nb_ctx *c, double t);
 // k_correct.cu

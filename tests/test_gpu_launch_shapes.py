@@ -36,3 +36,34 @@ def test_automatic_shape_matches_oracle(prec, n, n_act):
     kap = O.evaluate_kappa(m, x, v, a, eps, act) if prec else (None,) * 3
     for gq, rq, kq in zip(got, ref, kap):
         assert check_parity(min(prec, 1), gq, rq, kq, tol_mixed=1e-6 if prec == 1 else 1e-12) <= 1.0
+
+
+# sizes at the edges of the tiles (256, 512, 768 particles), even and odd tile
+# counts, a last tile of one particle, and more than one batch of offsets
+@pytest.mark.parametrize("prec,n", [(1, 4096), (1, 5121), (1, 7000), (1, 8192), (1, 16129), (1, 70000)])
+def test_all_particles_matches_listed_particles(prec, n):
+    """evaluate(None) may take each unordered pair once; the same particles given as a device list do not.  Both
+    against the FP64 sums: the parity bound in units of sum_j |T_ij| on a sample, and the whole set to twice it."""
+    nb = nb_gpu()
+    import torch
+    eps = 1e-4
+    m, x, v = ni.plummer(n, 80, imf="salpeter")
+    a = ni.random_state(n, 81, scale=2.0)
+    if prec == 3:
+        m, x, v, a = (dw(q) for q in (m, x, v, a))
+    g = nb.NBody(m, x, v, eps, precision=prec, start_forces=False)
+    g.set_state({"a": a})
+    g.predict(0.0)
+    got = g.evaluate(None)
+    again = g.evaluate(np.arange(n, dtype=np.int32))
+    listed = [q.cpu().numpy() for q in g.evaluate(torch.arange(n, dtype=torch.int32, device="cuda"), out="device")]
+    kap = g.evaluate_kappa()
+    g.close()
+    tol = {0: 1e-13, 1: 1e-6, 3: 1e-12}[prec]
+    pick = np.unique(np.concatenate([np.arange(0, n, n // 61), [n - 1]])).astype(np.int32)
+    ref = O.evaluate(m, x, v, a, eps, pick)
+    okap = O.evaluate_kappa(m, x, v, a, eps, pick)
+    for gq, aq, lq, kq, rq, oq in zip(got, again, listed, kap, ref, okap):
+        np.testing.assert_array_equal(gq, aq)       # the same list: the same evaluation, deterministic
+        assert check_parity(1, gq[pick], rq, oq, tol_mixed=tol) <= 1.0
+        assert (np.abs(gq - lq).max(axis=1) / kq).max() <= 2 * tol
