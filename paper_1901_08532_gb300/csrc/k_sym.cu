@@ -48,18 +48,58 @@ struct SymArgs {
     size_t ns;       // T * B
 };
 
-// cp.async of one 32-bit word; bytes = 0 writes a zero.
+// Is offset d evaluated from tile b (for even T the last offset only from the
+// lower half)?
+__host__ __device__ __forceinline__ bool sym_job(int T, int b, int d) { return 2 * d != T || b < T / 2; }
+
+// What a block does: part h of the jobs (tile b, offsets of group g), as nit
+// j-tiles of SUB particles.  The last group of an even T may be launched for
+// the lower half of the tiles only.
+template <int B, int SUB>
+struct SymJob {
+    int b, da, part, subs, nit;
+    __device__ __forceinline__ explicit SymJob(const SymArgs &a)
+    {
+        b = blockIdx.x / a.parts % a.tiles;
+        da = a.d0 + blockIdx.x / a.parts / a.tiles * a.k;
+        const int db = min(a.d1, da + a.k);
+        subs = B / SUB / a.parts;
+        part = blockIdx.x % a.parts * subs * SUB;
+        nit = max(0, (sym_job(a.tiles, b, db - 1) ? db : db - 1) - da) * subs;
+    }
+    __device__ __forceinline__ int offset(int it) const { return da + it / subs; }
+    __device__ __forceinline__ int start(const SymArgs &a, int it) const  // first particle of j-tile it
+    {
+        const int c = b + offset(it);
+        return (c >= a.tiles ? c - a.tiles : c) * B + part + it % subs * SUB;
+    }
+    __device__ __forceinline__ size_t jslot(const SymArgs &a, int it) const
+    {
+        return static_cast<size_t>(offset(it) - a.d0) * 9 * a.ns + start(a, it);
+    }
+    __device__ __forceinline__ size_t islot(const SymArgs &a) const
+    {
+        return static_cast<size_t>(blockIdx.x / a.parts / a.tiles * a.parts + blockIdx.x % a.parts) * 9 * a.ns;
+    }
+};
+
+// cp.async of 4, 8 or 16 bytes; bytes = 0 writes zeros.
 __device__ __forceinline__ void cp_async4(void *dst, const void *src, uint32_t bytes)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(bytes)
                  : "memory");
 }
+__device__ __forceinline__ void cp_async8(void *dst, const void *src, uint32_t bytes)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-// Is offset d evaluated from tile b (for even T the last offset only from the
-// lower half)?
-__host__ __device__ __forceinline__ bool sym_job(int T, int b, int d) { return 2 * d != T || b < T / 2; }
 
 // ----------------------------------------------------------------- mixed
 
@@ -138,11 +178,7 @@ __global__ void __launch_bounds__(kMixedThreads, 2) sym_mixed_kernel(SymArgs a)
     float *jacc = sm + 2 * NCF * TH;         // [18][TH]: hi of the 9 sums, then lo
     float *iacc = jacc + 18 * TH;            // [2 KP][18][TH]
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    // block -> part h of the job (tile b, offsets of group g); the last group of
-    // an even T may be launched for the lower half of the tiles only
-    const int h = blockIdx.x % a.parts, b = blockIdx.x / a.parts % a.tiles, g = blockIdx.x / a.parts / a.tiles;
-    const int da = a.d0 + g * a.k, db = min(a.d1, da + a.k);
-    const int part = B / a.parts, subs = part / TH;  // j per job part, tiles of TH
+    const SymJob<B, TH> job(a);
     const float *jf = static_cast<const float *>(a.jb);
     const float2 eps2 = f2(static_cast<float>(a.eps2));
     constexpr int kRow[12] = {0, 1, 2, 4, 5, 6, 7, 8, 9, 10, 11, 12};
@@ -150,7 +186,7 @@ __global__ void __launch_bounds__(kMixedThreads, 2) sym_mixed_kernel(SymArgs a)
     float2 ni[KP][12], nmi[KP], pi[KP][9];
 #pragma unroll
     for (int p = 0; p < KP; ++p) {
-        const int i = b * B + (w * KP + p) * 64 + 2 * lane;
+        const int i = job.b * B + (w * KP + p) * 64 + 2 * lane;
         const int i0 = min(i, a.n - 1), i1 = min(i + 1, a.n - 1);
 #pragma unroll
         for (int q = 0; q < 12; ++q)
@@ -165,22 +201,13 @@ __global__ void __launch_bounds__(kMixedThreads, 2) sym_mixed_kernel(SymArgs a)
     for (int q = 0; q < 18; ++q)
         jacc[q * TH + tid] = 0.0f;
 
-    // the sub-tiles of this block's jobs in order: it -> (offset, sub-tile)
-    const int last = (db - 1 >= da && !sym_job(a.tiles, b, db - 1)) ? db - 1 : db;
-    const int nit = max(0, last - da) * subs;
-    auto tile_start = [&](int it) {
-        int c = b + da + it / subs;
-        if (c >= a.tiles)
-            c -= a.tiles;
-        return c * B + h * part + (it % subs) * TH;
-    };
-    if (nit > 0)
-        load_tile_mixed(a, tile, tile_start(0));
-    for (int it = 0; it < nit; ++it) {
+    if (job.nit > 0)
+        load_tile_mixed(a, tile, job.start(a, 0));
+    for (int it = 0; it < job.nit; ++it) {
         cp_async_wait_all();
         __syncthreads();
-        if (it + 1 < nit)
-            load_tile_mixed(a, tile + ((it + 1) & 1) * NCF * TH, tile_start(it + 1));
+        if (it + 1 < job.nit)
+            load_tile_mixed(a, tile + ((it + 1) & 1) * NCF * TH, job.start(a, it + 1));
         const float *s = tile + (it & 1) * NCF * TH;
         for (int st = 0; st < W; ++st) {
             const int sub = ((st + w) & (W - 1)) * 32;
@@ -237,27 +264,315 @@ __global__ void __launch_bounds__(kMixedThreads, 2) sym_mixed_kernel(SymArgs a)
                     }
             __syncthreads();
         }
-        const int d = da + it / subs;
-        float2 *pj = static_cast<float2 *>(a.pj) + static_cast<size_t>(d - a.d0) * 9 * a.ns + tile_start(it) + tid;
+        float2 *out = static_cast<float2 *>(a.pj) + job.jslot(a, it) + tid;
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
-            if (d > 0)
-                pj[q * a.ns] = make_float2(jacc[q * TH + tid], jacc[(9 + q) * TH + tid]);
+            if (job.offset(it) > 0)
+                out[q * a.ns] = make_float2(jacc[q * TH + tid], jacc[(9 + q) * TH + tid]);
             jacc[q * TH + tid] = 0.0f;
             jacc[(9 + q) * TH + tid] = 0.0f;
         }
     }
-    float2 *pi_out = static_cast<float2 *>(a.pi) + static_cast<size_t>(g * a.parts + h) * 9 * a.ns;
+    float2 *out = static_cast<float2 *>(a.pi) + job.islot(a);
 #pragma unroll
     for (int p = 0; p < KP; ++p) {
-        const int i = b * B + (w * KP + p) * 64 + 2 * lane;
+        const int i = job.b * B + (w * KP + p) * 64 + 2 * lane;
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
             const float *ia = iacc + (p * 36 + q) * TH + tid;
-            *reinterpret_cast<float4 *>(&pi_out[q * a.ns + i]) =
+            *reinterpret_cast<float4 *>(&out[q * a.ns + i]) =
                 make_float4(ia[0], ia[9 * TH], ia[18 * TH], ia[27 * TH]);
         }
     }
+}
+
+// -------------------------------------------------------------------- EX
+
+// Warps per block (W) sets the tile: 64 W particles, two per thread in the
+// lanes of the packed values.
+__host__ __device__ constexpr int ex_tile(int w) { return 64 * w; }
+
+// Both directions of the pairs of two i-particles with one j in double words
+// (pair_ex with the powers of q shared): ni the negated i-values, nmi the
+// negated masses.
+__device__ __forceinline__ void pair_ex_sym(const float2 (&c)[NCX], const ExI<float2> &ni,
+                                            const ff::FF<float2> &nmi, const ff::FF<float2> &eps2,
+                                            ff::FF<float2> (&pi)[9], ff::FF<float2> (&pj)[9])
+{
+    using F = ff::FF<float2>;
+    F r[3], dv[3], da[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        r[k] = ff::add_accurate(F{c[k], c[3 + k]}, ni.x[k]);  // close pairs cancel
+        dv[k] = ff::add(F{c[6 + k], c[9 + k]}, ni.v[k]);
+        da[k] = ff::add(F{c[12 + k], c[15 + k]}, ni.a[k]);
+    }
+    const F R = ff::mad(r[0], r[0], ff::mad(r[1], r[1], ff::mad(r[2], r[2], eps2)));
+    const F rv = ff::mad(r[0], dv[0], ff::mad(r[1], dv[1], ff::mul(r[2], dv[2])));
+    const F sv = ff::mad(r[0], da[0], ff::mad(r[1], da[1], ff::mad(r[2], da[2],
+                 ff::mad(dv[0], dv[0], ff::mad(dv[1], dv[1], ff::sqr(dv[2]))))));
+    const F q = ff::rsqrt(R, rsqrt_est_v(R.h));
+    const F q2 = ff::sqr(q);
+    const F q3 = ff::mul(q, q2);
+    const F mu = ff::mul(F{c[18], c[19]}, q3), nu = ff::mul(nmi, q3);
+    const F al = ff::mul(rv, q2);
+    const F be = ff::mad(al, al, ff::mul(sv, q2));
+    const float2 m3 = f2(-3.0f), two = f2(2.0f);
+    const F na3 = ff::mul(al, m3);
+    const F na6 = {ff::mul(na3.h, two), ff::mul(na3.l, two)};  // exact doubling
+    const F nb3 = ff::mul(be, m3);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const F u = ff::mad(na3, r[k], dv[k]);
+        const F w = ff::mad(na6, u, ff::mad(nb3, r[k], da[k]));
+        ff::accumulate_mul(pi[k], mu, r[k]);
+        ff::accumulate_mul(pj[k], nu, r[k]);
+        ff::accumulate_mul(pi[3 + k], mu, u);
+        ff::accumulate_mul(pj[3 + k], nu, u);
+        ff::accumulate_mul(pi[6 + k], mu, w);
+        ff::accumulate_mul(pj[6 + k], nu, w);
+    }
+}
+
+// Bound by the FP32 pipe like the ordinary EX kernel; eight warps of 238
+// registers fill an SM, and the tile shrinks with W for small systems.
+// Double-word sums run over at most 64 terms in each half of a packed value, as
+// in the ordinary kernel; its RMS error is 0.95-1.0 of that kernel's.
+// All particles, ordinary kernel -> this one: 2000 81 -> 72 us, 4096 268 -> 207,
+// 16384 3.84 -> 2.58 ms, 40000 23.7 -> 15.0 ms (1.07e11 interactions/s).  Below
+// about 1800 particles the ordinary kernel is faster.
+template <int W>
+__global__ void __launch_bounds__(32 * W, 8 / W) sym_ex_kernel(SymArgs a)
+{
+    using F = ff::FF<float2>;
+    constexpr int TH = 32 * W, B = ex_tile(W);
+    extern __shared__ __align__(16) float sm[];
+    float *tile = sm;                 // [2][NCX][TH]
+    float *jacc = sm + 2 * NCX * TH;  // [18][TH]: high parts of the 9 sums, then low parts
+    float *iacc = jacc + 18 * TH;     // [2][18][TH]
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const SymJob<B, TH> job(a);
+    const float *jf = static_cast<const float *>(a.jb);
+    const float e2h = __double2float_rn(a.eps2);
+    const F eps2 = {f2(e2h), f2(__double2float_rn(a.eps2 - static_cast<double>(e2h)))};
+
+    const int i = job.b * B + w * 64 + 2 * lane;
+    const int i0 = min(i, a.n - 1), i1 = min(i + 1, a.n - 1);
+    auto neg = [&](int row) { return make_float2(-jf[row * a.np + i0], -jf[row * a.np + i1]); };
+    ExI<float2> ni;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        ni.x[k] = {neg(k), neg(3 + k)};
+        ni.v[k] = {neg(6 + k), neg(9 + k)};
+        ni.a[k] = {neg(12 + k), neg(15 + k)};
+    }
+    F nmi = {neg(18), neg(19)};
+    if (i >= a.n) nmi.h.x = nmi.l.x = 0.0f;
+    if (i + 1 >= a.n) nmi.h.y = nmi.l.y = 0.0f;
+    F pi[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+        pi[q] = {f2(0.0f), f2(0.0f)};
+    for (int q = 0; q < 36; ++q)
+        iacc[q * TH + tid] = 0.0f;
+    for (int q = 0; q < 18; ++q)
+        jacc[q * TH + tid] = 0.0f;
+
+    auto load = [&](int it) {
+        float *dst = tile + (it & 1) * NCX * TH;
+        const int j = job.start(a, it) + tid, jc = min(j, a.n - 1);  // beyond the end: no mass
+#pragma unroll
+        for (int r = 0; r < NCX; ++r)
+            cp_async4(dst + r * TH + tid, jf + r * a.np + jc, r >= 18 && j >= a.n ? 0u : 4u);
+        cp_async_commit();
+    };
+    // acc (h, l in shared memory, ld floats apart) += t
+    auto into = [](float *h, int ld, float th, float tl) {
+        ff::FF<float> s = {h[0], h[ld]};
+        ff::accumulate(s, ff::FF<float>{th, tl});
+        h[0] = s.h;
+        h[ld] = s.l;
+    };
+    if (job.nit > 0)
+        load(0);
+    for (int it = 0; it < job.nit; ++it) {
+        cp_async_wait_all();
+        __syncthreads();
+        if (it + 1 < job.nit)
+            load(it + 1);
+        const float *s = tile + (it & 1) * NCX * TH;
+        for (int st = 0; st < W; ++st) {
+            const int sub = ((st + w) & (W - 1)) * 32;
+            F pj[9];
+#pragma unroll
+            for (int q = 0; q < 9; ++q)
+                pj[q] = {f2(0.0f), f2(0.0f)};
+#pragma unroll 1
+            for (int step = 0; step < 32; ++step) {
+                const float *sj = s + sub + ((lane + step) & 31);
+                float2 c[NCX];
+#pragma unroll
+                for (int r = 0; r < NCX; ++r)
+                    c[r] = f2(sj[r * TH]);
+                pair_ex_sym(c, ni, nmi, eps2, pi, pj);
+#pragma unroll
+                for (int q = 0; q < 9; ++q) {
+                    pj[q].h.x = __shfl_sync(0xffffffffu, pj[q].h.x, lane + 1);
+                    pj[q].h.y = __shfl_sync(0xffffffffu, pj[q].h.y, lane + 1);
+                    pj[q].l.x = __shfl_sync(0xffffffffu, pj[q].l.x, lane + 1);
+                    pj[q].l.y = __shfl_sync(0xffffffffu, pj[q].l.y, lane + 1);
+                }
+            }
+            // double-word sums of 32 terms on each half of the j-side ...
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+                into(jacc + q * TH + sub + lane, 9 * TH, pj[q].h.x, pj[q].l.x);
+                into(jacc + q * TH + sub + lane, 9 * TH, pj[q].h.y, pj[q].l.y);
+            }
+            // ... and of 64 on the i-side (32 in a one-warp block)
+            if (W == 1 || (st & 1))
+#pragma unroll
+                for (int q = 0; q < 9; ++q) {
+                    into(iacc + q * TH + tid, 9 * TH, pi[q].h.x, pi[q].l.x);
+                    into(iacc + (18 + q) * TH + tid, 9 * TH, pi[q].h.y, pi[q].l.y);
+                    pi[q] = {f2(0.0f), f2(0.0f)};
+                }
+            __syncthreads();
+        }
+        float2 *out = static_cast<float2 *>(a.pj) + job.jslot(a, it) + tid;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            if (job.offset(it) > 0)
+                out[q * a.ns] = make_float2(jacc[q * TH + tid], jacc[(9 + q) * TH + tid]);
+            jacc[q * TH + tid] = 0.0f;
+            jacc[(9 + q) * TH + tid] = 0.0f;
+        }
+    }
+    float2 *out = static_cast<float2 *>(a.pi) + job.islot(a);
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+        *reinterpret_cast<float4 *>(&out[q * a.ns + i]) =
+            make_float4(iacc[q * TH + tid], iacc[(9 + q) * TH + tid], iacc[(18 + q) * TH + tid],
+                        iacc[(27 + q) * TH + tid]);
+}
+
+// ------------------------------------------------------------------ FP64
+
+// One i-particle per thread; the j-tile is 5 rows of 16-byte records.
+__device__ __forceinline__ void pair_fp64_sym(const double2 (&c)[5], const double (&xi)[9], double nmi, double eps2,
+                                              double (&pi)[9], double (&pj)[9])
+{
+    const double dx = c[0].x - xi[0], dy = c[0].y - xi[1], dz = c[1].x - xi[2];
+    const double dvx = c[2].x - xi[3], dvy = c[2].y - xi[4], dvz = c[3].x - xi[5];
+    const double dax = c[3].y - xi[6], day = c[4].x - xi[7], daz = c[4].y - xi[8];
+    const double r2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, eps2)));
+    const double rv = fma(dx, dvx, fma(dy, dvy, dz * dvz));
+    const double sv = fma(dx, dax, fma(dy, day, fma(dz, daz, fma(dvx, dvx, fma(dvy, dvy, dvz * dvz)))));
+    const double q = nbk::rsqrt_fp64(r2);
+    const double q2 = q * q, q3 = q * q2;
+    const double mu = c[1].y * q3, nu = nmi * q3;
+    const double al = rv * q2;
+    const double be = fma(al, al, sv * q2);
+    const double a3 = 3.0 * al, a6 = 6.0 * al, b3 = 3.0 * be;
+    const double ux = fma(-a3, dx, dvx), uy = fma(-a3, dy, dvy), uz = fma(-a3, dz, dvz);
+    const double wx = fma(-a6, ux, fma(-b3, dx, dax));
+    const double wy = fma(-a6, uy, fma(-b3, dy, day));
+    const double wz = fma(-a6, uz, fma(-b3, dz, daz));
+    const double t[9] = {dx, dy, dz, ux, uy, uz, wx, wy, wz};
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        pi[k] = fma(mu, t[k], pi[k]);
+        pj[k] = fma(nu, t[k], pj[k]);
+    }
+}
+
+// Bound by the FP64 pipe (94 % of 2 operations per clock and SM): 63 operations
+// per unordered pair for 106, so loads and shuffles cost nothing.  One warp per
+// scheduler fills the pipe; W = 1 and 2 give small systems enough blocks.
+// All particles, ordinary kernel -> this one: 1000 114 -> 96 us, 2000 402 ->
+// 275, 4096 1.58 -> 0.98 ms, 8191 6.24 -> 3.87, 30000 84.9 -> 50.3 ms
+// (1.79e10 interactions/s).  Below about 900 particles the ordinary kernel is
+// faster.
+template <int W>
+__global__ void __launch_bounds__(32 * W) sym_fp64_kernel(SymArgs a)
+{
+    constexpr int TH = 32 * W;
+    __shared__ __align__(16) double2 tile[2][5][TH];
+    __shared__ double jacc[9][TH];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const SymJob<TH, TH> job(a);
+    const double2 *jb = static_cast<const double2 *>(a.jb);
+    const int i = job.b * TH + tid;
+    double xi[9], nmi, acc[9], pi[9];
+    {
+        const int ic = min(i, a.n - 1);
+        const double2 r0 = jb[ic], r1 = jb[a.np + ic], r2 = jb[2 * a.np + ic], r3 = jb[3 * a.np + ic],
+                      r4 = jb[4 * a.np + ic];
+        xi[0] = r0.x; xi[1] = r0.y; xi[2] = r1.x;
+        xi[3] = r2.x; xi[4] = r2.y; xi[5] = r3.x;
+        xi[6] = r3.y; xi[7] = r4.x; xi[8] = r4.y;
+        nmi = i < a.n ? -r1.y : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        acc[q] = pi[q] = 0.0;
+        jacc[q][tid] = 0.0;
+    }
+    auto load = [&](int it) {
+        double2 (&dst)[5][TH] = tile[it & 1];
+        const int j = job.start(a, it) + tid, jc = min(j, a.n - 1);
+#pragma unroll
+        for (int r = 0; r < 5; ++r)
+            if (r != 1)
+                cp_async16(&dst[r][tid], jb + r * a.np + jc);
+        const double2 *zm = jb + a.np + jc;  // beyond the end: the last particle without its mass
+        cp_async8(&dst[1][tid].x, &zm->x, 8u);
+        cp_async8(&dst[1][tid].y, &zm->y, j >= a.n ? 0u : 8u);
+        cp_async_commit();
+    };
+    if (job.nit > 0)
+        load(0);
+    for (int it = 0; it < job.nit; ++it) {
+        cp_async_wait_all();
+        __syncthreads();
+        if (it + 1 < job.nit)
+            load(it + 1);
+        const double2 (&s)[5][TH] = tile[it & 1];
+        for (int st = 0; st < W; ++st) {
+            const int sub = ((st + w) & (W - 1)) * 32;
+            double pj[9];
+#pragma unroll
+            for (int q = 0; q < 9; ++q)
+                pj[q] = 0.0;
+#pragma unroll 1
+            for (int step = 0; step < 32; ++step) {
+                const int e = sub + ((lane + step) & 31);
+                const double2 c[5] = {s[0][e], s[1][e], s[2][e], s[3][e], s[4][e]};
+                pair_fp64_sym(c, xi, nmi, a.eps2, pi, pj);
+#pragma unroll
+                for (int q = 0; q < 9; ++q)
+                    pj[q] = __shfl_sync(0xffffffffu, pj[q], lane + 1);
+            }
+#pragma unroll
+            for (int q = 0; q < 9; ++q)
+                jacc[q][sub + lane] += pj[q];
+            __syncthreads();
+        }
+        // two-level summation: the j-tile's sums, then the running totals
+        double *out = static_cast<double *>(a.pj) + job.jslot(a, it) + tid;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            acc[q] += pi[q];
+            pi[q] = 0.0;
+            if (job.offset(it) > 0)
+                out[q * a.ns] = jacc[q][tid];
+            jacc[q][tid] = 0.0;
+        }
+    }
+    double *out = static_cast<double *>(a.pi) + job.islot(a) + i;
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+        out[q * a.ns] = acc[q];
 }
 
 // ------------------------------------------------------------------- fold
@@ -274,6 +589,51 @@ struct FoldFF {
     }
     __device__ __forceinline__ double total() const { return static_cast<double>(h) + static_cast<double>(l); }
 };
+
+// FP64 totals: of double words (EX) or doubles.
+struct FoldEx {
+    using Part = float2;
+    double s = 0.0;
+    __device__ __forceinline__ void add(float2 v) { s += static_cast<double>(v.x) + static_cast<double>(v.y); }
+    __device__ __forceinline__ double total() const { return s; }
+};
+// FP64 slots enter a compensated total (the rounding errors of a plain chain over
+// the T slots would exceed those of the ordinary kernel's sums: at 30000
+// particles 2.3e-16 of sum_j |A_ij| RMS against 0.7e-16).
+struct Fold64 {
+    using Part = double;
+    double s = 0.0, e = 0.0;
+    __device__ __forceinline__ void add(double v)
+    {
+        const double t = s + v, b = t - s;
+        e += (s - (t - b)) + (v - b);
+        s = t;
+    }
+    __device__ __forceinline__ double total() const { return s + e; }
+};
+
+template <class F, int U>
+__device__ __forceinline__ void add_all(F &f, const typename F::Part (&v)[U])
+{
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        f.add(v[u]);
+}
+template <int U>
+__device__ __forceinline__ void add_all(Fold64 &f, const double (&v)[U])
+{
+    // pairwise among themselves, compensated into the total
+    double t[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        t[u] = v[u];
+#pragma unroll
+    for (int h = U / 2; h > 0; h /= 2)
+#pragma unroll
+        for (int u = 0; u < h; ++u)
+            t[u] += t[u + h];
+    f.add(t[0]);
+}
 
 // out[q][p] (+)= the i-slots in order, then the j-slots in order of the offset.
 template <class F>
@@ -300,9 +660,7 @@ __global__ void __launch_bounds__(256) fold_kernel(const typename F::Part *pi, i
 #pragma unroll
         for (int u = 0; u < U; ++u)
             v[u] = src[(s + u) * step];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            f.add(v[u]);
+        add_all(f, v);
     }
     for (; s < nslots; ++s)
         f.add(src[s * step]);
@@ -314,9 +672,7 @@ __global__ void __launch_bounds__(256) fold_kernel(const typename F::Part *pi, i
 #pragma unroll
         for (int u = 0; u < U; ++u)
             v[u] = src[(d - d0 + u) * step];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            f.add(v[u]);
+        add_all(f, v);
     }
     for (; d < db; ++d)
         f.add(src[(d - d0) * step]);
@@ -324,39 +680,50 @@ __global__ void __launch_bounds__(256) fold_kernel(const typename F::Part *pi, i
     *o = first ? f.total() : *o + f.total();
 }
 
-size_t mixed_smem(int kp) { return sizeof(float) * kMixedThreads * (2 * NCF + 18 + 36 * kp); }
+constexpr size_t mixed_smem(int kp) { return sizeof(float) * kMixedThreads * (2 * NCF + 18 + 36 * kp); }
+constexpr size_t ex_smem(int w) { return sizeof(float) * 32 * w * (2 * NCX + 18 + 36); }
 
-}  // namespace
-
-// ------------------------------------------------------------------- plan
-
-// The kernels of a precision: particles per tile, threads, bytes of a partial
-// sum, and the measured rate with the chip full in unordered pairs per
-// microsecond and SM.
+// A kernel of a precision: particles per tile, threads, bytes of a partial sum,
+// dynamic shared memory, the measured rate with the chip full in unordered pairs
+// per microsecond and SM, and the jobs an SM needs for that rate.
 struct SymKind {
-    int kp, tile, threads, bytes;
-    double rate;
+    void (*kernel)(SymArgs);
+    int tile, threads, bytes;
+    size_t smem;
+    double rate, fill;
 };
 
-constexpr SymKind kMixedKinds[] = {{3, mixed_tile(3), kMixedThreads, 8, 3170.0},
-                                   {2, mixed_tile(2), kMixedThreads, 8, 2750.0},
-                                   {1, mixed_tile(1), kMixedThreads, 8, 2200.0}};
+const SymKind kKinds[] = {
+    {sym_mixed_kernel<3>, mixed_tile(3), kMixedThreads, 8, mixed_smem(3), 3170.0, 1.12},
+    {sym_mixed_kernel<2>, mixed_tile(2), kMixedThreads, 8, mixed_smem(2), 2750.0, 1.12},
+    {sym_mixed_kernel<1>, mixed_tile(1), kMixedThreads, 8, mixed_smem(1), 2200.0, 1.12},
+    {sym_ex_kernel<4>, ex_tile(4), 128, 8, ex_smem(4), 360.0, 1.3},
+    {sym_ex_kernel<2>, ex_tile(2), 64, 8, ex_smem(2), 355.0, 2.6},
+    {sym_ex_kernel<1>, ex_tile(1), 32, 8, ex_smem(1), 345.0, 5.2},
+    {sym_fp64_kernel<4>, 128, 128, 8, 0, 60.0, 1.05},
+    {sym_fp64_kernel<2>, 64, 64, 8, 0, 59.5, 2.1},
+    {sym_fp64_kernel<1>, 32, 32, 8, 0, 58.5, 4.2},
+};
+
+// Kinds of a precision: [first, first + 3).
+int first_kind(int precision) { return nb_fp32_eval(precision) ? 0 : precision == NB_EX ? 3 : 6; }
 
 // Tiles x groups of the offsets [d0, d1), without the upper half of the tiles
 // where the last group is the offset T / 2 alone.
-static int64_t sym_jobs(int64_t T, int64_t d0, int64_t d1, int64_t k)
+int64_t sym_jobs(int64_t T, int64_t d0, int64_t d1, int64_t k)
 {
     const int64_t groups = (d1 - d0 + k - 1) / k;
     return T * groups - (2 * (d1 - 1) == T && (d1 - d0 - 1) % k == 0 ? T / 2 : 0);
 }
 
 // The estimate behind a plan: the SM with the most jobs works through them at
-// the kernel's full rate (one block of four warps reaches 88 % of it), plus a
-// fixed part per job and launch and the traffic of the slots.  Within 5 % of
-// the measured times of the plans it chooses from 4096 to 524288 particles;
-// the next best plans lie within 2 % there.
-static void plan_kind(const SymKind &kd, int kind, int64_t n, int sms, SymPlan &best)
+// the kernel's full rate (with fewer than `fill` jobs as long as with that
+// many), plus a fixed part per job and launch and the traffic of the slots.
+// Mixed: within 5 % of the measured times of the plans it chooses from 4096 to
+// 524288 particles; the next best plans lie within 2 % there.
+void plan_kind(int kind, int64_t n, int sms, SymPlan &best)
 {
+    const SymKind &kd = kKinds[kind];
     const int64_t T = (n + kd.tile - 1) / kd.tile, D = T / 2 + 1;
     const double slot = 9.0 * kd.bytes * static_cast<double>(T * kd.tile);
     const int64_t slots = std::max<int64_t>(2, static_cast<int64_t>(kSymSlotBytes / slot));
@@ -373,9 +740,9 @@ static void plan_kind(const SymKind &kd, int kind, int64_t n, int sms, SymPlan &
             nd = (D + batches - 1) / batches;
             const int64_t groups = (nd + k - 1) / k;
             const int64_t jobs = (T * nd - (T % 2 == 0 && batches == 1 ? T / 2 : 0)) * parts / k;
-            const int64_t each = (jobs + sms - 1) / sms;
+            const double each = static_cast<double>((jobs + sms - 1) / sms) + (k > 1 ? 0.5 : 0.05);
             const double pairs = static_cast<double>(kd.tile) * kd.tile * std::min<int64_t>(k, nd) / parts;
-            const double us = batches * ((each > 1 ? each + (k > 1 ? 0.5 : 0.05) : 1.12) * (pairs / kd.rate + 1.0) + 5.0 +
+            const double us = batches * (std::max(each, kd.fill) * (pairs / kd.rate + 1.0) + 5.0 +
                                          (nd + groups * parts) * slot * 2.0 / 6e6);
             if (us < best.us) {
                 best.us = us;
@@ -391,33 +758,32 @@ static void plan_kind(const SymKind &kd, int kind, int64_t n, int sms, SymPlan &
         }
 }
 
+}  // namespace
+
 SymPlan nb_sym_plan(int precision, int64_t n, int sms)
 {
     SymPlan best;
-    if (nb_fp32_eval(precision))
-        for (int q = 0; q < 3; ++q)
-            plan_kind(kMixedKinds[q], q, n, sms, best);
+    for (int q = 0; q < 3; ++q)
+        plan_kind(first_kind(precision) + q, n, sms, best);
     return best;
-}
-
-template <typename K>
-static cudaError_t allow_smem(K kernel, size_t bytes)
-{
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
 }
 
 cudaError_t nb_sym_smem_setup()
 {
-    cudaError_t e;
-    if ((e = allow_smem(sym_mixed_kernel<1>, mixed_smem(1))) != cudaSuccess) return e;
-    if ((e = allow_smem(sym_mixed_kernel<2>, mixed_smem(2))) != cudaSuccess) return e;
-    return allow_smem(sym_mixed_kernel<3>, mixed_smem(3));
+    for (const SymKind &kd : kKinds)
+        if (kd.smem > 0) {
+            const cudaError_t e = cudaFuncSetAttribute(kd.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       static_cast<int>(kd.smem));
+            if (e != cudaSuccess)
+                return e;
+        }
+    return cudaSuccess;
 }
 
 cudaError_t nb_launch_sym(int precision, const SymPlan &pl, const void *jb, size_t np, int n, double eps2,
                           void *work, double *out, size_t ostride, cudaStream_t stream, int *launches)
 {
-    const SymKind &kd = kMixedKinds[pl.kind];
+    const SymKind &kd = kKinds[pl.kind];
     SymArgs a;
     a.jb = jb;
     a.np = np;
@@ -433,17 +799,24 @@ cudaError_t nb_launch_sym(int precision, const SymPlan &pl, const void *jb, size
     for (int d0 = 0; d0 < D; d0 += pl.nd) {
         a.d0 = d0;
         a.d1 = std::min(D, d0 + pl.nd);
+        const int64_t jobs = sym_jobs(pl.T, a.d0, a.d1, pl.k);
         const int groups = (a.d1 - a.d0 + pl.k - 1) / pl.k;
-        const unsigned grid = static_cast<unsigned>(sym_jobs(pl.T, a.d0, a.d1, pl.k) * pl.parts);
-        const size_t smem = mixed_smem(kd.kp);
-        if (kd.kp == 3) sym_mixed_kernel<3><<<grid, kd.threads, smem, stream>>>(a);
-        else if (kd.kp == 2) sym_mixed_kernel<2><<<grid, kd.threads, smem, stream>>>(a);
-        else sym_mixed_kernel<1><<<grid, kd.threads, smem, stream>>>(a);
-        fold_kernel<FoldFF><<<dim3((n + 255) / 256, 9), 256, 0, stream>>>(
-            static_cast<const float2 *>(a.pi), groups * pl.parts,
-            static_cast<int>(sym_jobs(pl.T, a.d0, a.d1, pl.k) / pl.T) * pl.parts,
-            static_cast<const float2 *>(a.pj), a.d0, a.d1,
-            a.ns, pl.T, kd.tile, n, out, ostride, d0 == 0);
+        const int upper = static_cast<int>(jobs / pl.T) * pl.parts;  // i-slots of the upper half of the tiles
+        kd.kernel<<<static_cast<unsigned>(jobs * pl.parts), kd.threads, kd.smem, stream>>>(a);
+        const dim3 grid((n + 255) / 256, 9);
+        auto fold = [&](auto f) {
+            using F = decltype(f);
+            using P = typename F::Part;
+            fold_kernel<F><<<grid, 256, 0, stream>>>(static_cast<const P *>(a.pi), groups * pl.parts, upper,
+                                                     static_cast<const P *>(a.pj), a.d0, a.d1, a.ns, pl.T,
+                                                     kd.tile, n, out, ostride, d0 == 0);
+        };
+        if (precision == NB_FP64)
+            fold(Fold64{});
+        else if (precision == NB_EX)
+            fold(FoldEx{});
+        else
+            fold(FoldFF{});
         *launches += 2;
     }
     return cudaGetLastError();

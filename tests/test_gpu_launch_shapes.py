@@ -38,9 +38,11 @@ def test_automatic_shape_matches_oracle(prec, n, n_act):
         assert check_parity(min(prec, 1), gq, rq, kq, tol_mixed=1e-6 if prec == 1 else 1e-12) <= 1.0
 
 
-# sizes at the edges of the tiles (256, 512, 768 particles), even and odd tile
-# counts, a last tile of one particle, and more than one batch of offsets
-@pytest.mark.parametrize("prec,n", [(1, 4096), (1, 5121), (1, 7000), (1, 8192), (1, 16129), (1, 70000)])
+# sizes at the edges of the tiles (mixed 256, 512, 768 particles, EX 64 to 256, FP64 32 to 128), even and odd
+# tile counts, a last tile of one particle, several parts of a j-tile and several offsets per block
+@pytest.mark.parametrize("prec,n", [(1, 4096), (1, 5121), (1, 7000), (1, 8192), (1, 16129), (1, 70000),
+                                    (0, 1000), (0, 1025), (0, 2049), (0, 4096), (0, 8193),
+                                    (3, 2000), (3, 3001), (3, 4096), (3, 8193), (3, 16641)])
 def test_all_particles_matches_listed_particles(prec, n):
     """evaluate(None) may take each unordered pair once; the same particles given as a device list do not.  Both
     against the FP64 sums: the parity bound in units of sum_j |T_ij| on a sample, and the whole set to twice it."""
