@@ -1,22 +1,22 @@
 // Energy and angular momentum of the current state (paper, section 3 item 3:
 // both are evaluated on the device and checked periodically; Eq. 1 defines
 // their relative errors).  FP64 throughout, deterministic: per-block sums in
-// a fixed tree order, then one block adds the block sums in index order.
+// a fixed tree order, then one block adds the block sums in a fixed order.
 //   E_kin = sum 1/2 m_i |v_i|^2
 //   E_pot = -sum_{i<j} m_i m_j / sqrt(|r_ij|^2 + eps^2)
-//         = 1/2 sum_i m_i phi_i,  phi_i = -sum_{j != i} m_j / sqrt(...)
 //   L     = sum m_i x_i cross v_i,  and sum m_i |x_i cross v_i|
+#include <algorithm>
+
 #include "nb_internal.cuh"
 
 namespace {
 
 constexpr int kT = 256;
-constexpr int kTile = 256;
 
-template <int NV>
+template <int NV, int TH>
 __device__ void block_sum(double (&v)[NV], double *out)
 {
-    __shared__ double s[NV][kT / 32];
+    __shared__ double s[NV][TH / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
@@ -31,52 +31,76 @@ __device__ void block_sum(double (&v)[NV], double *out)
 #pragma unroll
         for (int q = 0; q < NV; ++q) {
             double x = 0.0;
-            for (int w = 0; w < kT / 32; ++w)
+            for (int w = 0; w < TH / 32; ++w)
                 x += s[q][w];
             out[q] = x;
         }
     }
 }
 
-__global__ void __launch_bounds__(kT) energy_kernel(const double *st, const double *m, int n,
-                                                    double eps2, double *blocksums)
+// 1 / sqrt(x): the refined FP32 estimate in its range, the library functions
+// beyond (positions 1e19 and more apart, infinities, NaN).
+__device__ __forceinline__ double inv_sqrt(double x)
 {
-    __shared__ double sx[kTile], sy[kTile], sz[kTile], sm[kTile];
+    if (__double2hiint(x) >= (1023 + 126) << 20 || __double2hiint(x) < 0)
+        return 1.0 / sqrt(x);
+    return nbk::rsqrt_fp64(x);
+}
+
+// Every unordered pair once: the particles form T tiles of B, a block takes the
+// pairs of tile b with the tiles b + d (mod T) for its k offsets d of
+// 0 .. T/2 (for even T the last offset counts from the lower half of the tiles
+// only; d = 0 is the tile with itself, in ordered pairs at half weight).  128
+// threads: B = 128 gives each an i-particle, B = 32 each warp a quarter of
+// the j-tile, for systems that would otherwise leave SMs idle.
+// Bound by the FP64 pipe: 12 operations per pair (was sqrt and a division for
+// every ordered pair, on n / 256 blocks).  nb_energy, 1000 particles 1603 -> 42 us,
+// 8192 12.96 -> 0.79 ms, 131072 827 -> 186 ms.
+constexpr int kET = 128;
+
+template <int B>
+__global__ void __launch_bounds__(kET) energy_kernel(const double *st, const double *m, int n, double eps2, int T,
+                                                     int k, double *blocksums)
+{
+    constexpr int S = kET / B;  // threads that share an i-particle
+    __shared__ double sx[B], sy[B], sz[B], sm[B];
     const size_t N = static_cast<size_t>(n);
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = blockIdx.x, da = blockIdx.y * k, db = min(T / 2 + 1, da + k);
+    const int i = b * B + threadIdx.x % B, part = threadIdx.x / B;
     const bool valid = i < n;
-    const int ii = valid ? i : 0;
-    const double xi = st[(F_X * 3 + 0) * N + ii], yi = st[(F_X * 3 + 1) * N + ii],
-                 zi = st[(F_X * 3 + 2) * N + ii];
+    const int ii = valid ? i : n - 1;
+    const double *x = st + F_X * 3 * N, *v = st + F_V * 3 * N;
+    const double xi = x[ii], yi = x[N + ii], zi = x[2 * N + ii];
     double phi = 0.0;
-    for (int j0 = 0; j0 < n; j0 += kTile) {
+    for (int d = da; d < db; ++d) {
+        if (2 * d == T && b >= T / 2)
+            break;
+        const int c = b + d < T ? b + d : b + d - T;
         __syncthreads();
-        for (int q = threadIdx.x; q < kTile; q += blockDim.x) {
-            const int j = j0 + q;
-            const bool ok = j < n;
-            sx[q] = ok ? st[(F_X * 3 + 0) * N + j] : 0.0;
-            sy[q] = ok ? st[(F_X * 3 + 1) * N + j] : 0.0;
-            sz[q] = ok ? st[(F_X * 3 + 2) * N + j] : 0.0;
-            sm[q] = ok ? m[j] : 0.0;
+        if (threadIdx.x < B) {
+            const int j = c * B + threadIdx.x, jj = min(j, n - 1);
+            sx[threadIdx.x] = x[jj];
+            sy[threadIdx.x] = x[N + jj];
+            sz[threadIdx.x] = x[2 * N + jj];
+            sm[threadIdx.x] = j < n ? m[j] : 0.0;
         }
         __syncthreads();
-        const int len = min(kTile, n - j0);
-        double part = 0.0;
-        for (int q = 0; q < len; ++q) {
+        double s = 0.0;
+#pragma unroll 4
+        for (int q = part * (B / S); q < (part + 1) * (B / S); ++q) {
             const double dx = sx[q] - xi, dy = sy[q] - yi, dz = sz[q] - zi;
-            const double r = sqrt(fma(dx, dx, fma(dy, dy, fma(dz, dz, eps2))));
-            part += (j0 + q == i) ? 0.0 : sm[q] / r;
+            const double r = inv_sqrt(fma(dx, dx, fma(dy, dy, fma(dz, dz, eps2))));
+            s = (d == 0 && c * B + q == i) ? s : fma(sm[q], r, s);
         }
-        phi += part;
+        phi += d == 0 ? 0.5 * s : s;
     }
-    double v[2] = {0.0, 0.0};
+    double w[2] = {0.0, 0.0};
     if (valid) {
-        const double vx = st[(F_V * 3 + 0) * N + i], vy = st[(F_V * 3 + 1) * N + i],
-                     vz = st[(F_V * 3 + 2) * N + i];
-        v[0] = 0.5 * m[i] * fma(vx, vx, fma(vy, vy, vz * vz));
-        v[1] = -0.5 * m[i] * phi;
+        w[1] = -m[i] * phi;
+        if (da == 0 && part == 0)
+            w[0] = 0.5 * m[i] * fma(v[i], v[i], fma(v[N + i], v[N + i], v[2 * N + i] * v[2 * N + i]));
     }
-    block_sum<2>(v, blocksums + 2 * blockIdx.x);
+    block_sum<2, kET>(w, blocksums + 2 * (static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x));
 }
 
 __global__ void __launch_bounds__(kT) angmom_kernel(const double *st, const double *m, int n,
@@ -96,19 +120,22 @@ __global__ void __launch_bounds__(kT) angmom_kernel(const double *st, const doub
         v[2] = m[i] * lz;
         v[3] = m[i] * sqrt(lx * lx + ly * ly + lz * lz);
     }
-    block_sum<4>(v, blocksums + 4 * blockIdx.x);
+    block_sum<4, kT>(v, blocksums + 4 * blockIdx.x);
 }
 
-// Sum nv interleaved block sums in block order (one thread per value).
-__global__ void final_sum_kernel(const double *blocksums, int nblocks, int nv, double *out)
+// Sum nv interleaved block sums in a fixed order (one block).
+template <int NV>
+__global__ void __launch_bounds__(kT) final_sum_kernel(const double *blocksums, int nblocks, double *out)
 {
-    const int q = threadIdx.x;
-    if (q >= nv)
-        return;
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b)
-        s += blocksums[b * nv + q];
-    out[q] = s;
+    double v[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q)
+        v[q] = 0.0;
+    for (int b = threadIdx.x; b < nblocks; b += kT)
+#pragma unroll
+        for (int q = 0; q < NV; ++q)
+            v[q] += blocksums[static_cast<size_t>(b) * NV + q];
+    block_sum<NV, kT>(v, out);
 }
 
 cudaError_t ensure_red(nb_ctx *c, size_t doubles)
@@ -130,12 +157,20 @@ cudaError_t ensure_red(nb_ctx *c, size_t doubles)
 cudaError_t nb_launch_energy(nb_ctx *c, double *out_dev)
 {
     const int n = static_cast<int>(c->n);
-    const int nb = (n + kT - 1) / kT;
+    // 32-particle tiles below 6144 particles (1024: 528 blocks instead of 36)
+    const int B = n < 6144 ? 32 : kET;
+    const int T = (n + B - 1) / B, D = T / 2 + 1;
+    // offsets per block: about 16384 blocks at most
+    const int groups = std::max(1, std::min(D, 16384 / T)), k = (D + groups - 1) / groups;
+    const dim3 grid(T, (D + k - 1) / k);
+    const int nb = static_cast<int>(grid.x * grid.y);
     cudaError_t e = ensure_red(c, static_cast<size_t>(2) * nb);
     if (e != cudaSuccess)
         return e;
-    energy_kernel<<<nb, kT, 0, c->stream>>>(c->st, c->m, n, c->eps * c->eps, c->red);
-    final_sum_kernel<<<1, 32, 0, c->stream>>>(c->red, nb, 2, out_dev);
+    const double eps2 = c->eps * c->eps;
+    if (B == 32) energy_kernel<32><<<grid, kET, 0, c->stream>>>(c->st, c->m, n, eps2, T, k, c->red);
+    else energy_kernel<kET><<<grid, kET, 0, c->stream>>>(c->st, c->m, n, eps2, T, k, c->red);
+    final_sum_kernel<2><<<1, kT, 0, c->stream>>>(c->red, nb, out_dev);
     c->launches += 2;
     return cudaGetLastError();
 }
@@ -149,7 +184,7 @@ cudaError_t nb_launch_angmom(nb_ctx *c, double *out_dev)
     if (e != cudaSuccess)
         return e;
     angmom_kernel<<<nb, kT, 0, c->stream>>>(c->st, c->m, n, c->red);
-    final_sum_kernel<<<1, 32, 0, c->stream>>>(c->red, nb, 4, out_dev);
+    final_sum_kernel<4><<<1, kT, 0, c->stream>>>(c->red, nb, out_dev);
     c->launches += 2;
     return cudaGetLastError();
 }
