@@ -442,6 +442,20 @@ nb_status nb_pairs_fp64_adjoint(int64_t n, const double *m, const double *x, con
                                 const double *gjerk, const double *gsnap, double *gx, double *gv,
                                 double *ga, double *gm, void *stream);
 
+/* Bytes of device workspace nb_pairs_fp64_adjoint_work needs for n particles
+ * (0 where it runs as nb_pairs_fp64_adjoint; caller allocated, 256-byte
+ * aligned, reusable between calls on one stream). */
+size_t nb_pairs_adjoint_workspace_bytes(int64_t n);
+
+/* nb_pairs_fp64_adjoint with a workspace for partial sums, so that each
+ * unordered pair is taken once (about half the time from some 700 particles
+ * on; no atomics, deterministic).  work = NULL is nb_pairs_fp64_adjoint.
+ * Errors: NB_EINVAL, NB_ECUDA. */
+nb_status nb_pairs_fp64_adjoint_work(int64_t n, const double *m, const double *x, const double *v,
+                                     const double *a, double eps, const double *gacc,
+                                     const double *gjerk, const double *gsnap, double *gx, double *gv,
+                                     double *ga, double *gm, void *work, void *stream);
+
 /* The O(N) stages of a fixed-step Hermite trajectory (section 3: predictor
  * and corrector around the evaluation; every particle on the shared step of
  * section 3 item 3) and their adjoints, for differentiating trajectories.

@@ -110,6 +110,11 @@ _lib.nb_pairs_fp64.restype = C.c_int
 _lib.nb_pairs_fp64_adjoint.argtypes = [C.c_int64, _vp, _vp, _vp, _vp, C.c_double, _vp, _vp, _vp,
                                        _vp, _vp, _vp, _vp, _vp]
 _lib.nb_pairs_fp64_adjoint.restype = C.c_int
+_lib.nb_pairs_adjoint_workspace_bytes.argtypes = [C.c_int64]
+_lib.nb_pairs_adjoint_workspace_bytes.restype = C.c_size_t
+_lib.nb_pairs_fp64_adjoint_work.argtypes = [C.c_int64, _vp, _vp, _vp, _vp, C.c_double, _vp, _vp, _vp,
+                                            _vp, _vp, _vp, _vp, _vp, _vp]
+_lib.nb_pairs_fp64_adjoint_work.restype = C.c_int
 _lib.nb_traj_predict.argtypes = [C.c_int64, C.c_double] + [_vp] * 9 + [_vp]
 _lib.nb_traj_predict_adjoint.argtypes = [C.c_int64, C.c_double] + [_vp] * 9 + [_vp]
 _lib.nb_traj_correct.argtypes = [C.c_int64, C.c_double] + [_vp] * 11 + [_vp]
@@ -137,7 +142,7 @@ EXPORTED = ("nb_config_default", "nb_init", "nb_predict", "nb_get_predicted", "n
             "nb_ensemble_set_shape", "nb_ensemble_get_shape", "nb_ensemble_run", "nb_ensemble_get_state",
             "nb_ensemble_stats", "nb_ensemble_set_log", "nb_ensemble_get_log",
             "nb_ensemble_last_error", "nb_ensemble_free", "nb_pairs_workspace_bytes", "nb_pairs_fp64",
-            "nb_pairs_fp64_adjoint", "nb_traj_predict", "nb_traj_predict_adjoint", "nb_traj_correct",
+            "nb_pairs_fp64_adjoint", "nb_pairs_adjoint_workspace_bytes", "nb_pairs_fp64_adjoint_work", "nb_traj_predict", "nb_traj_predict_adjoint", "nb_traj_correct",
             "nb_traj_correct_adjoint", "nb_peak_probe")
 
 PROBE_KINDS = ("ffma", "ffma2", "dfma", "rsqrt", "rcp", "ffma2+rsqrt", "ffma2+rsqrt_noftz",

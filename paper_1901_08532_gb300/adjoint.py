@@ -6,7 +6,7 @@ interpolation's crackle; every particle active, as in the paper's shared
 time step) as a torch.autograd.Function: its forward runs the library's
 predictor, FP64 all-pairs evaluation and corrector kernels, and its backward
 the library's hand-written adjoints of the three (nb_traj_correct_adjoint,
-nb_pairs_fp64_adjoint, nb_traj_predict_adjoint) through the C-ABI; torch
+nb_pairs_fp64_adjoint_work, nb_traj_predict_adjoint) through the C-ABI; torch
 only allocates the tensors.  `PairSums` is the evaluation alone (used for
 the start-up).  `torch.utils.checkpoint` keeps only every
 `checkpoint`-th state, recomputing each segment in the backward pass.
@@ -20,17 +20,23 @@ from torch.utils.checkpoint import checkpoint
 
 from . import NB_OK, NBError, lib
 
-_work_cache: dict = {}
+
+def _workspace(nbytes: int, device) -> torch.Tensor:
+    """Device memory for one call on the current stream, from torch's caching allocator: it goes back with the call's
+    last use of it in stream order, so calls on different streams never share it."""
+    return torch.empty(max(1, int(nbytes)), dtype=torch.uint8, device=device)
 
 
-def _workspace(n: int, device) -> torch.Tensor:
-    key = (n, device)
-    w = _work_cache.get(key)
-    if w is None:
-        nbytes = int(lib().nb_pairs_workspace_bytes(n))
-        w = torch.empty(nbytes, dtype=torch.uint8, device=device)
-        _work_cache[key] = w
-    return w
+def _forward_work(n: int, device) -> torch.Tensor:
+    return _workspace(lib().nb_pairs_workspace_bytes(n), device)
+
+
+def _pairs_adjoint(n, args, eps, outs, device, stream):
+    """The pair sums' adjoint with its workspace (none for small systems)."""
+    work = _workspace(lib().nb_pairs_adjoint_workspace_bytes(n), device)
+    _check(lib().nb_pairs_fp64_adjoint_work(n, *[_ptr(t) for t in args[:4]], float(eps),
+                                            *[_ptr(t) for t in args[4:]], *[_ptr(t) for t in outs], _ptr(work),
+                                            stream))
 
 
 def _ptr(t: torch.Tensor):
@@ -54,8 +60,9 @@ class PairSums(torch.autograd.Function):
         jerk = torch.empty_like(x)
         snap = torch.empty_like(x)
         stream = torch.cuda.current_stream(x.device).cuda_stream
+        work = _forward_work(n, x.device)
         _check(lib().nb_pairs_fp64(n, _ptr(m), _ptr(x), _ptr(v), _ptr(a), float(eps), _ptr(acc),
-                                   _ptr(jerk), _ptr(snap), _ptr(_workspace(n, x.device)),
+                                   _ptr(jerk), _ptr(snap), _ptr(work),
                                    C.c_void_p(stream)))
         ctx.save_for_backward(m, x, v, a)
         ctx.eps = eps
@@ -72,9 +79,8 @@ class PairSums(torch.autograd.Function):
         gx, gv, ga = (torch.empty_like(x) for _ in range(3))
         gm = torch.empty_like(m)
         stream = torch.cuda.current_stream(x.device).cuda_stream
-        _check(lib().nb_pairs_fp64_adjoint(n, _ptr(m), _ptr(x), _ptr(v), _ptr(a), float(ctx.eps),
-                                           _ptr(g_acc), _ptr(g_jerk), _ptr(g_snap), _ptr(gx),
-                                           _ptr(gv), _ptr(ga), _ptr(gm), C.c_void_p(stream)))
+        _pairs_adjoint(n, (m, x, v, a, g_acc, g_jerk, g_snap), ctx.eps, (gx, gv, ga, gm), x.device,
+                       C.c_void_p(stream))
         return gm, gx, gv, ga, None
 
 
@@ -92,8 +98,9 @@ class HermiteStep(torch.autograd.Function):
         _check(lib().nb_traj_predict(n, float(h), *[_ptr(t) for t in (x, v, a, j, s, c, xp, vp, ap)],
                                      stream))
         A, J, S = (torch.empty_like(x) for _ in range(3))
+        work = _forward_work(n, x.device)
         _check(lib().nb_pairs_fp64(n, _ptr(m), _ptr(xp), _ptr(vp), _ptr(ap), float(eps), _ptr(A),
-                                   _ptr(J), _ptr(S), _ptr(_workspace(n, x.device)), stream))
+                                   _ptr(J), _ptr(S), _ptr(work), stream))
         x1, v1, c1 = (torch.empty_like(x) for _ in range(3))
         _check(lib().nb_traj_correct(n, float(h), *[_ptr(t) for t in (x, v, a, j, s, A, J, S, x1, v1,
                                                                         c1)], stream))
@@ -115,9 +122,7 @@ class HermiteStep(torch.autograd.Function):
                                                                           gSt)], stream))
         gxp, gvp, gap = (torch.empty_like(xp) for _ in range(3))
         gm = torch.empty_like(m)
-        _check(lib().nb_pairs_fp64_adjoint(n, _ptr(m), _ptr(xp), _ptr(vp), _ptr(ap), float(ctx.eps),
-                                           _ptr(gAt), _ptr(gJt), _ptr(gSt), _ptr(gxp), _ptr(gvp),
-                                           _ptr(gap), _ptr(gm), stream))
+        _pairs_adjoint(n, (m, xp, vp, ap, gAt, gJt, gSt), ctx.eps, (gxp, gvp, gap, gm), xp.device, stream)
         gc = torch.empty_like(xp)
         _check(lib().nb_traj_predict_adjoint(n, h, _ptr(gxp), _ptr(gvp), _ptr(gap), _ptr(gx), _ptr(gv),
                                              _ptr(ga), _ptr(gj), _ptr(gs), _ptr(gc), stream))

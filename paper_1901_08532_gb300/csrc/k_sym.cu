@@ -30,58 +30,11 @@
 #include "nb_device.cuh"
 #include "nb_ff.cuh"
 #include "nb_internal.cuh"
+#include "nb_sym.cuh"
 
 namespace {
 
 using namespace nbk;
-
-struct SymArgs {
-    const void *jb;  // predicted particles (the evaluation buffer's rows)
-    size_t np;       // row stride
-    int n;
-    int tiles;       // T
-    int d0, d1;      // offsets of this launch, [d0, d1)
-    int k;           // offsets per block
-    int parts;       // H, parts of a j-tile
-    double eps2;
-    void *pi, *pj;   // partial sums: [group * H + h][9][ns], [d - d0][9][ns]
-    size_t ns;       // T * B
-};
-
-// Is offset d evaluated from tile b (for even T the last offset only from the
-// lower half)?
-__host__ __device__ __forceinline__ bool sym_job(int T, int b, int d) { return 2 * d != T || b < T / 2; }
-
-// What a block does: part h of the jobs (tile b, offsets of group g), as nit
-// j-tiles of SUB particles.  The last group of an even T may be launched for
-// the lower half of the tiles only.
-template <int B, int SUB>
-struct SymJob {
-    int b, da, part, subs, nit;
-    __device__ __forceinline__ explicit SymJob(const SymArgs &a)
-    {
-        b = blockIdx.x / a.parts % a.tiles;
-        da = a.d0 + blockIdx.x / a.parts / a.tiles * a.k;
-        const int db = min(a.d1, da + a.k);
-        subs = B / SUB / a.parts;
-        part = blockIdx.x % a.parts * subs * SUB;
-        nit = max(0, (sym_job(a.tiles, b, db - 1) ? db : db - 1) - da) * subs;
-    }
-    __device__ __forceinline__ int offset(int it) const { return da + it / subs; }
-    __device__ __forceinline__ int start(const SymArgs &a, int it) const  // first particle of j-tile it
-    {
-        const int c = b + offset(it);
-        return (c >= a.tiles ? c - a.tiles : c) * B + part + it % subs * SUB;
-    }
-    __device__ __forceinline__ size_t jslot(const SymArgs &a, int it) const
-    {
-        return static_cast<size_t>(offset(it) - a.d0) * 9 * a.ns + start(a, it);
-    }
-    __device__ __forceinline__ size_t islot(const SymArgs &a) const
-    {
-        return static_cast<size_t>(blockIdx.x / a.parts / a.tiles * a.parts + blockIdx.x % a.parts) * 9 * a.ns;
-    }
-};
 
 // cp.async of 4, 8 or 16 bytes; bytes = 0 writes zeros.
 __device__ __forceinline__ void cp_async4(void *dst, const void *src, uint32_t bytes)
@@ -590,142 +543,62 @@ struct FoldFF {
     __device__ __forceinline__ double total() const { return static_cast<double>(h) + static_cast<double>(l); }
 };
 
-// FP64 totals: of double words (EX) or doubles.
+// FP64 totals of double words (EX).
 struct FoldEx {
     using Part = float2;
     double s = 0.0;
     __device__ __forceinline__ void add(float2 v) { s += static_cast<double>(v.x) + static_cast<double>(v.y); }
     __device__ __forceinline__ double total() const { return s; }
 };
-// FP64 slots enter a compensated total (the rounding errors of a plain chain over
-// the T slots would exceed those of the ordinary kernel's sums: at 30000
-// particles 2.3e-16 of sum_j |A_ij| RMS against 0.7e-16).
-struct Fold64 {
-    using Part = double;
-    double s = 0.0, e = 0.0;
-    __device__ __forceinline__ void add(double v)
-    {
-        const double t = s + v, b = t - s;
-        e += (s - (t - b)) + (v - b);
-        s = t;
-    }
-    __device__ __forceinline__ double total() const { return s + e; }
-};
-
-template <class F, int U>
-__device__ __forceinline__ void add_all(F &f, const typename F::Part (&v)[U])
-{
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-        f.add(v[u]);
-}
-template <int U>
-__device__ __forceinline__ void add_all(Fold64 &f, const double (&v)[U])
-{
-    // pairwise among themselves, compensated into the total
-    double t[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-        t[u] = v[u];
-#pragma unroll
-    for (int h = U / 2; h > 0; h /= 2)
-#pragma unroll
-        for (int u = 0; u < h; ++u)
-            t[u] += t[u + h];
-    f.add(t[0]);
-}
-
-// out[q][p] (+)= the i-slots in order, then the j-slots in order of the offset.
+// out[q][p] (+)= the slots of a batch of offsets.
 template <class F>
 __global__ void __launch_bounds__(256) fold_kernel(const typename F::Part *pi, int nslots, int upper,
                                                    const typename F::Part *pj, int d0, int d1, size_t ns,
                                                    int T, int B, int n, double *out, size_t ostride, int first)
 {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    const int q = blockIdx.y;
     if (p >= n)
         return;
-    constexpr int U = 8;  // slots in flight
-    F f;
-    const size_t step = 9 * ns;
-    const typename F::Part *src = pi + q * ns + p;
-    // tile c takes j-sums at every offset but 0, and at d = T/2 only in the
-    // upper half, which has `upper` i-slots
-    const int c = p / B;
-    if (c >= T / 2)
-        nslots = upper;
-    int s = 0;
-    for (; s + U <= nslots; s += U) {
-        typename F::Part v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            v[u] = src[(s + u) * step];
-        add_all(f, v);
-    }
-    for (; s < nslots; ++s)
-        f.add(src[s * step]);
-    const int da = max(d0, 1), db = (2 * (d1 - 1) == T && c < T / 2) ? d1 - 1 : d1;
-    src = pj + q * ns + p;
-    int d = da;
-    for (; d + U <= db; d += U) {
-        typename F::Part v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            v[u] = src[(d - d0 + u) * step];
-        add_all(f, v);
-    }
-    for (; d < db; ++d)
-        f.add(src[(d - d0) * step]);
-    double *o = out + q * ostride + p;
-    *o = first ? f.total() : *o + f.total();
+    const double s = fold_slots<F, 9>(pi, nslots, upper, pj, d0, d1, ns, T, B, blockIdx.y, p);
+    double *o = out + blockIdx.y * ostride + p;
+    *o = first ? s : *o + s;
 }
 
 constexpr size_t mixed_smem(int kp) { return sizeof(float) * kMixedThreads * (2 * NCF + 18 + 36 * kp); }
 constexpr size_t ex_smem(int w) { return sizeof(float) * 32 * w * (2 * NCX + 18 + 36); }
 
-// A kernel of a precision: particles per tile, threads, bytes of a partial sum,
-// dynamic shared memory, the measured rate with the chip full in unordered pairs
-// per microsecond and SM, and the jobs an SM needs for that rate.
 struct SymKind {
     void (*kernel)(SymArgs);
-    int tile, threads, bytes;
     size_t smem;
-    double rate, fill;
+    SymShape shape;
 };
 
 const SymKind kKinds[] = {
-    {sym_mixed_kernel<3>, mixed_tile(3), kMixedThreads, 8, mixed_smem(3), 3170.0, 1.12},
-    {sym_mixed_kernel<2>, mixed_tile(2), kMixedThreads, 8, mixed_smem(2), 2750.0, 1.12},
-    {sym_mixed_kernel<1>, mixed_tile(1), kMixedThreads, 8, mixed_smem(1), 2200.0, 1.12},
-    {sym_ex_kernel<4>, ex_tile(4), 128, 8, ex_smem(4), 360.0, 1.3},
-    {sym_ex_kernel<2>, ex_tile(2), 64, 8, ex_smem(2), 355.0, 2.6},
-    {sym_ex_kernel<1>, ex_tile(1), 32, 8, ex_smem(1), 345.0, 5.2},
-    {sym_fp64_kernel<4>, 128, 128, 8, 0, 60.0, 1.05},
-    {sym_fp64_kernel<2>, 64, 64, 8, 0, 59.5, 2.1},
-    {sym_fp64_kernel<1>, 32, 32, 8, 0, 58.5, 4.2},
+    {sym_mixed_kernel<3>, mixed_smem(3), {mixed_tile(3), kMixedThreads, 72, 3170.0, 1.12}},
+    {sym_mixed_kernel<2>, mixed_smem(2), {mixed_tile(2), kMixedThreads, 72, 2750.0, 1.12}},
+    {sym_mixed_kernel<1>, mixed_smem(1), {mixed_tile(1), kMixedThreads, 72, 2200.0, 1.12}},
+    {sym_ex_kernel<4>, ex_smem(4), {ex_tile(4), 128, 72, 360.0, 1.3}},
+    {sym_ex_kernel<2>, ex_smem(2), {ex_tile(2), 64, 72, 355.0, 2.6}},
+    {sym_ex_kernel<1>, ex_smem(1), {ex_tile(1), 32, 72, 345.0, 5.2}},
+    {sym_fp64_kernel<4>, 0, {128, 128, 72, 60.0, 1.05}},
+    {sym_fp64_kernel<2>, 0, {64, 64, 72, 59.5, 2.1}},
+    {sym_fp64_kernel<1>, 0, {32, 32, 72, 58.5, 4.2}},
 };
 
 // Kinds of a precision: [first, first + 3).
 int first_kind(int precision) { return nb_fp32_eval(precision) ? 0 : precision == NB_EX ? 3 : 6; }
 
-// Tiles x groups of the offsets [d0, d1), without the upper half of the tiles
-// where the last group is the offset T / 2 alone.
-int64_t sym_jobs(int64_t T, int64_t d0, int64_t d1, int64_t k)
-{
-    const int64_t groups = (d1 - d0 + k - 1) / k;
-    return T * groups - (2 * (d1 - 1) == T && (d1 - d0 - 1) % k == 0 ? T / 2 : 0);
-}
+}  // namespace
 
 // The estimate behind a plan: the SM with the most jobs works through them at
 // the kernel's full rate (with fewer than `fill` jobs as long as with that
 // many), plus a fixed part per job and launch and the traffic of the slots.
 // Mixed: within 5 % of the measured times of the plans it chooses from 4096 to
 // 524288 particles; the next best plans lie within 2 % there.
-void plan_kind(int kind, int64_t n, int sms, SymPlan &best)
+void nb_sym_plan_shape(const SymShape &kd, int kind, int64_t n, int sms, SymPlan &best)
 {
-    const SymKind &kd = kKinds[kind];
     const int64_t T = (n + kd.tile - 1) / kd.tile, D = T / 2 + 1;
-    const double slot = 9.0 * kd.bytes * static_cast<double>(T * kd.tile);
+    const double slot = static_cast<double>(kd.bytes) * static_cast<double>(T * kd.tile);
     const int64_t slots = std::max<int64_t>(2, static_cast<int64_t>(kSymSlotBytes / slot));
     const int subs = kd.tile / kd.threads;
     for (const int k : {1, 2, 4, 8})
@@ -758,13 +631,11 @@ void plan_kind(int kind, int64_t n, int sms, SymPlan &best)
         }
 }
 
-}  // namespace
-
 SymPlan nb_sym_plan(int precision, int64_t n, int sms)
 {
     SymPlan best;
     for (int q = 0; q < 3; ++q)
-        plan_kind(first_kind(precision) + q, n, sms, best);
+        nb_sym_plan_shape(kKinds[first_kind(precision) + q].shape, first_kind(precision) + q, n, sms, best);
     return best;
 }
 
@@ -783,7 +654,8 @@ cudaError_t nb_sym_smem_setup()
 cudaError_t nb_launch_sym(int precision, const SymPlan &pl, const void *jb, size_t np, int n, double eps2,
                           void *work, double *out, size_t ostride, cudaStream_t stream, int *launches)
 {
-    const SymKind &kd = kKinds[pl.kind];
+    const SymKind &kind = kKinds[pl.kind];
+    const SymShape &kd = kind.shape;
     SymArgs a;
     a.jb = jb;
     a.np = np;
@@ -794,7 +666,7 @@ cudaError_t nb_launch_sym(int precision, const SymPlan &pl, const void *jb, size
     a.eps2 = eps2;
     a.ns = pl.ns;
     a.pi = work;
-    a.pj = static_cast<unsigned char *>(work) + pl.pi_slots * 9 * pl.ns * kd.bytes;
+    a.pj = static_cast<unsigned char *>(work) + pl.pi_slots * pl.ns * kd.bytes;
     const int D = pl.T / 2 + 1;
     for (int d0 = 0; d0 < D; d0 += pl.nd) {
         a.d0 = d0;
@@ -802,7 +674,7 @@ cudaError_t nb_launch_sym(int precision, const SymPlan &pl, const void *jb, size
         const int64_t jobs = sym_jobs(pl.T, a.d0, a.d1, pl.k);
         const int groups = (a.d1 - a.d0 + pl.k - 1) / pl.k;
         const int upper = static_cast<int>(jobs / pl.T) * pl.parts;  // i-slots of the upper half of the tiles
-        kd.kernel<<<static_cast<unsigned>(jobs * pl.parts), kd.threads, kd.smem, stream>>>(a);
+        kind.kernel<<<static_cast<unsigned>(jobs * pl.parts), kd.threads, kind.smem, stream>>>(a);
         const dim3 grid((n + 255) / 256, 9);
         auto fold = [&](auto f) {
             using F = decltype(f);
