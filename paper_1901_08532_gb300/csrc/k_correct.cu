@@ -1,5 +1,5 @@
 // Corrector stage and time-step selection (paper, section 3 and section 3
-// item 3), one thread per active particle, FP64:
+// item 3), three threads per active particle, FP64:
 //   * 6th-order Hermite corrector (the two-point quadrature with a, a', a''
 //     at both ends, exact for a(t) of degree <= 5), v first, then x;
 //   * crackle, pop and the 5th derivative of a at the end of the step from
@@ -30,17 +30,21 @@ struct CorrectArgs {
     nb_ctl *ctl;
 };
 
-__global__ void __launch_bounds__(128) correct_kernel(CorrectArgs a)
+// 32 particles per block, one component per warp (nb_correct.cuh).
+constexpr int kCorrectThreads = 96;
+
+__global__ void __launch_bounds__(kCorrectThreads) correct_kernel(CorrectArgs a)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= a.n_act)
-        return;
-    double f[9];
+    __shared__ nbk::CorrectScratch sh;
+    const int k = blockIdx.x * 32 + (threadIdx.x & 31), d = threadIdx.x >> 5;
+    const bool valid = k < a.n_act;
+    double f[3] = {0.0, 0.0, 0.0};
+    if (valid)
 #pragma unroll
-    for (int q = 0; q < 9; ++q)
-        f[q] = a.anew[q * (size_t)a.ostride + k];
-    nbk::correct_particle_fp64(a.st, a.t, a.dt, static_cast<size_t>(a.n), a.act[k], a.t1, f, a.eta,
-                               a.dt_min, a.dt_max, a.dt_shared, a.ctl, a.noise);
+        for (int q = 0; q < 3; ++q)
+            f[q] = a.anew[(3 * q + d) * (size_t)a.ostride + k];
+    nbk::correct_group_fp64(a.st, a.t, a.dt, static_cast<size_t>(a.n), valid ? a.act[k] : 0, valid, a.t1, f, a.eta,
+                            a.dt_min, a.dt_max, a.dt_shared, a.ctl, a.noise, sh);
 }
 
 // Start-up (nb_init): pass 0 stores a and jerk of the first evaluation (made
@@ -157,7 +161,7 @@ cudaError_t nb_launch_correct(nb_ctx *c, double t1, int n_act)
     a.dt_max = c->cfg.dt_max;
     a.dt_shared = c->cfg.dt_shared;
     a.ctl = c->ctl;
-    correct_kernel<<<(n_act + 127) / 128, 128, 0, c->stream>>>(a);
+    correct_kernel<<<(n_act + 31) / 32, kCorrectThreads, 0, c->stream>>>(a);
     c->launches += 1;
     return cudaGetLastError();
 }

@@ -49,32 +49,32 @@ __global__ void __launch_bounds__(256) predict_kernel(const double *__restrict__
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     const double d = q[3 * g + k];
-                    const float h = __double2float_rn(d);
+                    const float h = nbk::to_float(d);
                     jf32[(6 * g + k) * npad + i] = h;
-                    jf32[(6 * g + 3 + k) * npad + i] = __double2float_rn(d - static_cast<double>(h));
+                    jf32[(6 * g + 3 + k) * npad + i] = nbk::to_float(d - nbk::to_double(h));
                 }
-            const float mh = __double2float_rn(mi);
+            const float mh = nbk::to_float(mi);
             jf32[18 * npad + i] = mh;
-            jf32[19 * npad + i] = __double2float_rn(mi - static_cast<double>(mh));
+            jf32[19 * npad + i] = nbk::to_float(mi - nbk::to_double(mh));
         } else if (jf32) {
             const bool drop_lo = mode == kModeSp;
             float h[3], l[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                h[k] = __double2float_rn(p[k].x);
-                l[k] = drop_lo ? 0.0f : __double2float_rn(p[k].x - static_cast<double>(h[k]));
+                h[k] = nbk::to_float(p[k].x);
+                l[k] = drop_lo ? 0.0f : nbk::to_float(p[k].x - nbk::to_double(h[k]));
             }
             jf32[0 * npad + i] = h[0];
             jf32[1 * npad + i] = h[1];
             jf32[2 * npad + i] = h[2];
-            jf32[3 * npad + i] = __double2float_rn(mi);
+            jf32[3 * npad + i] = nbk::to_float(mi);
             jf32[4 * npad + i] = l[0];
             jf32[5 * npad + i] = l[1];
             jf32[6 * npad + i] = l[2];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                jf32[(7 + k) * npad + i] = __double2float_rn(p[k].v);
-                jf32[(10 + k) * npad + i] = __double2float_rn(p[k].a);
+                jf32[(7 + k) * npad + i] = nbk::to_float(p[k].v);
+                jf32[(10 + k) * npad + i] = nbk::to_float(p[k].a);
             }
         }
     }

@@ -10,14 +10,22 @@
 //             the earliest t_i + dt_i and lists the particles that reach it;
 //             after a grid barrier all blocks read the same minima and counts
 //             and take the same decision;
-//   evaluate  every block predicts its slice into shared memory (chunk by
-//             chunk, the layout of the evaluation buffer of the precision),
-//             predicts the active particles itself, and sums the active set
-//             against its slice; partial sums go to global memory;
+//   evaluate  every block predicts its slice and the active particles into
+//             shared memory (chunk by chunk, the layout of the evaluation
+//             buffer of the precision) and sums the active set against its
+//             slice; partial sums go to global memory;
 //   correct   after a second grid barrier the block that owns an active
-//             particle adds the partial sums of all blocks in block order and
-//             applies the FP64 corrector and step selection (the same device
-//             function as the corrector kernel).
+//             particle adds the partial sums of all blocks in a fixed order
+//             and applies the FP64 corrector and step selection (the same
+//             device function as the corrector kernel).
+// What bounds a step is latency: two barriers, the L2 round trips between
+// them, and above all serial chains of FP64 instructions, each of which holds
+// a scheduler's pipe for 64 clocks for a warp however few of its threads are
+// active.  So FP64 work is spread over the block's four warps (prediction
+// and corrector by component, sums over lanes and over blocks by value, each
+// output a short chain of one thread), and comparisons use integers.  Time
+// per step with about 13 active particles, before -> after: FP64 N = 1024
+// 39.2 -> 18.1 us, EX N = 8192 46.1 -> 20.7 us, mixed N = 65536 58.0 -> 31.6 us.
 // It returns to the host when the next active set holds more than
 // kStepSmall particles (the host then runs that step with the tuned
 // evaluation kernels), when the next block time passes t_end, or after an
@@ -38,8 +46,14 @@ namespace {
 
 using namespace nbk;
 
-constexpr int kStepThreads = 128;
+constexpr int kQ = 2;            // blocks of the grid per thread in the step decision
 constexpr int kStepSmall = 128;  // active sets up to this size are stepped on the device
+// Particles per block at least (small systems: fewer blocks), and the slice from
+// which a block has 256 threads instead of 128: more warps predict a long
+// slice, fewer make every sum over lanes and blocks shorter (us a step, 128 / 256
+// threads: EX N = 8192 20.7 / 21.6, EX 20000 30.8 / 26.8, mixed 65536
+// 38.5 / 31.6; FP64 N = 1024 with 8 and 16 particles per block 18.1 and 19.4).
+constexpr int kSliceFp64 = 8, kSliceFp32 = 16, kSliceWide = 96;
 constexpr int kChunkCap = 1024;  // j-records per shared-memory chunk
 
 struct StepOut {
@@ -56,10 +70,10 @@ struct StepArgs {
     const double *m;
     double eps2, eta, dt_min, dt_max, dt_shared, t_end, noise;
     int drop_lo;        // single-precision control: positions without their low part
-    double *bmin;       // [B] per-block earliest t_i + dt_i
+    unsigned long long *bmin;  // [B] per-block earliest t_i + dt_i, as bits
     int *bcnt;          // [B] particles reaching it
     int *cand;          // [B][kStepSmall] their indices, ascending
-    double *part;       // [B][kStepSmall][9] partial sums
+    double *part;       // [kStepSmall][9][B] partial sums
     int32_t *act;       // active set of the last step taken
     nb_ctl *ctl;
     StepOut *out;
@@ -71,17 +85,20 @@ struct StepArgs {
 // Bytes per j-record in shared memory: FP64 5 x 16, mixed 13 x 4, EX 20 x 4.
 __host__ __device__ constexpr int rec_bytes(int pr) { return pr == 0 ? 80 : (pr == 1 ? NCF * 4 : NCX * 4); }
 
-__device__ __forceinline__ double block_min_d(double v, double *red)
+// Block minimum of 64-bit values (non-negative doubles order like their bits).
+__device__ __forceinline__ unsigned long long block_min_u64(unsigned long long v, unsigned long long *red)
 {
-    for (int o = 16; o > 0; o >>= 1)
-        v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long u = __shfl_xor_sync(0xffffffffu, v, o);
+        v = u < v ? u : v;
+    }
     __syncthreads();
     if ((threadIdx.x & 31) == 0)
         red[threadIdx.x >> 5] = v;
     __syncthreads();
-    double r = red[0];
+    unsigned long long r = red[0];
     for (int q = 1; q < static_cast<int>(blockDim.x >> 5); ++q)
-        r = fmin(r, red[q]);
+        r = red[q] < r ? red[q] : r;
     return r;
 }
 
@@ -108,96 +125,78 @@ __device__ __forceinline__ int block_scan_excl(int v, int *red, int *total)
     return base + incl - v;
 }
 
-// The predicted record of particle i at time tp in the precision's layout:
-// FP64 5 double2 rows; mixed 13 FP32 rows (x_hi, m, x_lo, v, a; x_lo = 0 for
-// the single-precision control); EX 20 FP32 rows (hi then lo of x, v, a; m
-// hi, lo).  Rows go to rf[row * stride] (FP32 layouts) or rd[row * stride]
-// (FP64 layout).
+// Component d of the predicted record of particle i at time tp, in rows of
+// `stride` entries: FP64 10 rows x y z m vx vy vz ax ay az; mixed 13 FP32 rows
+// (x_hi, m, x_lo, v, a; x_lo = 0 for the single-precision control); EX 20 FP32
+// rows (hi then lo of x, v, a; m hi, lo).  d = 0 also stores the mass.
 template <int PR>
-__device__ __forceinline__ void predict_record(const StepArgs &a, int i, double tp, float *rf,
-                                               double2 *rd, int stride)
+__device__ __forceinline__ void predict_component(const StepArgs &a, int i, int d, double tp, void *rows, int stride)
 {
-    const size_t N = static_cast<size_t>(a.n);
-    const double d = tp - a.t[i];
-    Taylor p[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-        p[k] = taylor(a.st[(F_X * 3 + k) * N + i], a.st[(F_V * 3 + k) * N + i], a.st[(F_A * 3 + k) * N + i],
-                      a.st[(F_J * 3 + k) * N + i], a.st[(F_S * 3 + k) * N + i], a.st[(F_C * 3 + k) * N + i], d);
-    const double mi = a.m[i];
+    const size_t N = static_cast<size_t>(a.n), at = static_cast<size_t>(d) * N + i;
+    const double dt = tp - a.t[i];
+    const Taylor p = taylor(a.st[F_X * 3 * N + at], a.st[F_V * 3 * N + at], a.st[F_A * 3 * N + at],
+                            a.st[F_J * 3 * N + at], a.st[F_S * 3 * N + at], a.st[F_C * 3 * N + at], dt);
     if constexpr (PR == 0) {
-        rd[0] = make_double2(p[0].x, p[1].x);
-        rd[stride] = make_double2(p[2].x, mi);
-        rd[2 * stride] = make_double2(p[0].v, p[1].v);
-        rd[3 * stride] = make_double2(p[2].v, p[0].a);
-        rd[4 * stride] = make_double2(p[1].a, p[2].a);
+        double *r = static_cast<double *>(rows);
+        r[d * stride] = p.x;
+        r[(4 + d) * stride] = p.v;
+        r[(7 + d) * stride] = p.a;
+        if (d == 0)
+            r[3 * stride] = a.m[i];
     } else if constexpr (PR == 1) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const float h = __double2float_rn(p[k].x);
-            rf[k * stride] = h;
-            rf[(4 + k) * stride] = a.drop_lo ? 0.0f : __double2float_rn(p[k].x - static_cast<double>(h));
-            rf[(7 + k) * stride] = __double2float_rn(p[k].v);
-            rf[(10 + k) * stride] = __double2float_rn(p[k].a);
-        }
-        rf[3 * stride] = __double2float_rn(mi);
+        float *r = static_cast<float *>(rows);
+        const float h = to_float(p.x);
+        r[d * stride] = h;
+        r[(4 + d) * stride] = a.drop_lo ? 0.0f : to_float(p.x - to_double(h));
+        r[(7 + d) * stride] = to_float(p.v);
+        r[(10 + d) * stride] = to_float(p.a);
+        if (d == 0)
+            r[3 * stride] = to_float(a.m[i]);
     } else {
+        float *r = static_cast<float *>(rows);
+        const double q[3] = {p.x, p.v, p.a};
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const double q[3] = {p[k].x, p[k].v, p[k].a};
-#pragma unroll
-            for (int g = 0; g < 3; ++g) {
-                const float h = __double2float_rn(q[g]);
-                rf[(6 * g + k) * stride] = h;
-                rf[(6 * g + 3 + k) * stride] = __double2float_rn(q[g] - static_cast<double>(h));
-            }
+        for (int g = 0; g < 3; ++g) {
+            const float h = to_float(q[g]);
+            r[(6 * g + d) * stride] = h;
+            r[(6 * g + 3 + d) * stride] = to_float(q[g] - to_double(h));
         }
-        const float mh = __double2float_rn(mi);
-        rf[18 * stride] = mh;
-        rf[19 * stride] = __double2float_rn(mi - static_cast<double>(mh));
+        if (d == 0) {
+            const double mi = a.m[i];
+            const float mh = to_float(mi);
+            r[18 * stride] = mh;
+            r[19 * stride] = to_float(mi - to_double(mh));
+        }
     }
 }
 
-// i-values of active particle i (the same arithmetic as its j-record):
-// FP64 x, v, a; mixed 12 negated FP32 (x_hi, x_lo, v, a); EX 18 negated FP32
-// (hi then lo of x, v, a).  iv holds 9 doubles = 18 floats.
-template <int PR>
-__device__ __forceinline__ void ivalues(const StepArgs &a, int i, double tp, double *iv)
+__host__ __device__ constexpr int rows_of(int pr) { return pr == 0 ? 10 : pr == 1 ? NCF : NCX; }
+// Row entry size: double or float.
+__host__ __device__ constexpr int word_of(int pr) { return pr == 0 ? 8 : 4; }
+
+// v[0] + ... + v[n - 1] in four chains.
+__device__ __forceinline__ double sum4(const double *v, int n)
 {
-    if constexpr (PR == 0) {
-        double2 r[5];
-        predict_record<0>(a, i, tp, nullptr, r, 1);
-        iv[0] = r[0].x; iv[1] = r[0].y; iv[2] = r[1].x;
-        iv[3] = r[2].x; iv[4] = r[2].y; iv[5] = r[3].x;
-        iv[6] = r[3].y; iv[7] = r[4].x; iv[8] = r[4].y;
-    } else if constexpr (PR == 1) {
-        float r[NCF];
-        predict_record<1>(a, i, tp, r, nullptr, 1);
-        float *f = reinterpret_cast<float *>(iv);
-        constexpr int kRow[12] = {0, 1, 2, 4, 5, 6, 7, 8, 9, 10, 11, 12};
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int e = 0; e < n; e += 4)
 #pragma unroll
-        for (int q = 0; q < 12; ++q)
-            f[q] = -r[kRow[q]];
-    } else {
-        float r[NCX];
-        predict_record<2>(a, i, tp, r, nullptr, 1);
-        float *f = reinterpret_cast<float *>(iv);
-#pragma unroll
-        for (int q = 0; q < 18; ++q)
-            f[q] = -r[q];
-    }
+        for (int c = 0; c < 4; ++c)
+            if (e + c < n)
+                s[c] += v[e + c];
+    return (s[0] + s[1]) + (s[2] + s[3]);
 }
 
-// Partial sums of the K active particles (i-values iv) over the j of
-// [lo, hi), predicted to tp chunk by chunk into shared memory, written to
-// part[K][9].  L = T / K2 lanes per active particle (K2 the power of two
-// >= K) take every L-th j (pair of j in the FP32 precisions); lanes are
-// combined in a fixed order.
-template <int PR>
-__device__ void eval_slice(const StepArgs &a, int lo, int hi, double tp, int K, const double (*iv)[9],
-                           double *part, double (*wred)[9], unsigned char *smem)
+// Sums of the K active particles (listed in act) over the j of [lo, hi), all
+// predicted to tp, written to part[(k * 9 + q) * pstride].  L = T / K2 lanes per
+// active particle (K2 the power of two >= K) take every L-th j (pair of j in
+// the FP32 precisions); their sums meet in shared memory, where one thread per
+// value adds them in lane order.  rec: rows of the active particles; red: 9 T
+// 8-byte words.
+template <int PR, int T>
+__device__ void eval_slice(const StepArgs &a, int lo, int hi, double tp, int K, const int *act, void *rec,
+                           double *part, int pstride, double *red, unsigned char *smem)
 {
-    const int T = blockDim.x, tid = threadIdx.x;
+    const int tid = threadIdx.x;
     int K2 = 1;
     while (K2 < K)
         K2 <<= 1;
@@ -207,50 +206,72 @@ __device__ void eval_slice(const StepArgs &a, int lo, int hi, double tp, int K, 
     const int gi = valid ? g : 0;
     constexpr int cap = kChunkCap;
     float *sf = reinterpret_cast<float *>(smem);
-    double2 *sd = reinterpret_cast<double2 *>(smem);
+    double *sd = reinterpret_cast<double *>(smem);
     double acc[9];
-#pragma unroll
-    for (int q = 0; q < 9; ++q)
-        acc[q] = 0.0;
-    // FP32 precisions: packed pair sums, folded every 32 iterations
     float2 ni[12], pm[9];
     float ah[9], al[9];
     ExI<float2> nie;
     ff::FF<float2> px[9];
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
+        acc[q] = 0.0;
         pm[q] = f2(0.0f);
         ah[q] = al[q] = 0.0f;
         px[q] = {f2(0.0f), f2(0.0f)};
-    }
-    if (PR == 1) {
-        const float *f = reinterpret_cast<const float *>(iv[gi]);
-#pragma unroll
-        for (int q = 0; q < 12; ++q)
-            ni[q] = f2(f[q]);
-    } else if (PR == 2) {
-        const float *f = reinterpret_cast<const float *>(iv[gi]);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            nie.x[k] = {f2(f[k]), f2(f[3 + k])};
-            nie.v[k] = {f2(f[6 + k]), f2(f[9 + k])};
-            nie.a[k] = {f2(f[12 + k]), f2(f[15 + k])};
-        }
     }
     const float2 eps2f = f2(__double2float_rn(a.eps2));
     const float e2h = __double2float_rn(a.eps2);
     const ff::FF<float2> eps2x = {f2(e2h), f2(__double2float_rn(a.eps2 - static_cast<double>(e2h)))};
     int cnt = 0;
-    for (int b = lo; b < hi; b += cap) {
-        const int len = min(cap, hi - b);
-        for (int u = tid; u < len; u += T)
-            predict_record<PR>(a, b + u, tp, sf + u, sd + u, cap);
+    bool first = true, spilled = false;
+    for (int b = lo; b < hi || first; b += cap) {
+        const int len = max(0, min(cap, hi - b)), ka = first ? K : 0;
+        // the slice and, with the first chunk, the active particles: few of
+        // them by component, so that more warps share the FP64 chain; many
+        // whole (the five step factors once instead of three times)
+        const int m = len + ka, split = 2 * T >= 3 * m ? 3 : 1;
+        for (int u = tid; u < split * m; u += T) {
+            const int d0 = u / m, e = u - d0 * m;
+            const int i = e < len ? b + e : act[e - len];
+            unsigned char *rows = e < len ? smem + static_cast<size_t>(e) * word_of(PR)
+                                          : static_cast<unsigned char *>(rec) + static_cast<size_t>(e - len) * word_of(PR);
+            const int stride = e < len ? cap : kStepSmall;
+            if (split == 3)
+                predict_component<PR>(a, i, d0, tp, rows, stride);
+            else
+#pragma unroll
+                for (int d = 0; d < 3; ++d)
+                    predict_component<PR>(a, i, d, tp, rows, stride);
+        }
         __syncthreads();
+        if (first) {
+            if (PR == 1) {
+                const float *f = static_cast<const float *>(rec) + gi;
+                constexpr int kRow[12] = {0, 1, 2, 4, 5, 6, 7, 8, 9, 10, 11, 12};
+#pragma unroll
+                for (int q = 0; q < 12; ++q)
+                    ni[q] = f2(-f[kRow[q] * kStepSmall]);
+            } else if (PR == 2) {
+                const float *f = static_cast<const float *>(rec) + gi;
+                auto neg = [&](int row) { return f2(-f[row * kStepSmall]); };
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    nie.x[k] = {neg(k), neg(3 + k)};
+                    nie.v[k] = {neg(6 + k), neg(9 + k)};
+                    nie.a[k] = {neg(12 + k), neg(15 + k)};
+                }
+            }
+            first = false;
+        }
         if constexpr (PR == 0) {
-            const double *v = iv[gi];
-            for (int jj = lane; jj < len; jj += L)
-                pair_fp64(sd[jj], sd[cap + jj], sd[2 * cap + jj], sd[3 * cap + jj], sd[4 * cap + jj], v[0], v[1],
-                          v[2], v[3], v[4], v[5], v[6], v[7], v[8], a.eps2, acc);
+            const double *v = static_cast<const double *>(rec) + gi;
+            auto iv = [&](int row) { return v[row * kStepSmall]; };
+            for (int jj = lane; jj < len; jj += L) {
+                auto c = [&](int row) { return sd[row * cap + jj]; };
+                pair_fp64(make_double2(c(0), c(1)), make_double2(c(2), c(3)), make_double2(c(4), c(5)),
+                          make_double2(c(6), c(7)), make_double2(c(8), c(9)), iv(0), iv(1), iv(2), iv(4), iv(5), iv(6),
+                          iv(7), iv(8), iv(9), a.eps2, acc);
+            }
         } else {
             constexpr int NR = PR == 1 ? NCF : NCX;
             constexpr int mrow = PR == 1 ? 3 : 18;  // first mass row
@@ -285,73 +306,99 @@ __device__ void eval_slice(const StepArgs &a, int lo, int hi, double tp, int K, 
                         }
                     }
                     cnt = 0;
+                    spilled = true;
                 }
             }
         }
         __syncthreads();
     }
-    const int w = tid >> 5;
-    const int span = L < 32 ? L : 32;
-    if (PR == 1) {
+    // this thread's sums: doubles, or (hi, lo) words in the FP32 precisions
+    // (EX: the two halves of the packed sums joined by a double-word sum, and
+    // FP64 only where more than 32 iterations went to acc)
 #pragma unroll
-        for (int q = 0; q < 9; ++q) {
+    for (int q = 0; q < 9; ++q) {
+        if (PR == 0) {
+            red[tid * 9 + q] = acc[q];
+        } else if (PR == 1) {
             two_sum_acc(ah[q], al[q], __fadd_rn(pm[q].x, pm[q].y));
+            const int span = L < 32 ? L : 32;
             for (int o = span >> 1; o > 0; o >>= 1) {
                 const float oh = __shfl_xor_sync(0xffffffffu, ah[q], o);
                 const float ol = __shfl_xor_sync(0xffffffffu, al[q], o);
                 two_sum_acc(ah[q], al[q], oh);
                 al[q] = __fadd_rn(al[q], ol);
             }
-            acc[q] = static_cast<double>(ah[q]) + static_cast<double>(al[q]);
+            reinterpret_cast<float2 *>(red)[tid * 9 + q] = make_float2(ah[q], al[q]);
+        } else {
+            const ff::FF<float> x = {px[q].h.x, px[q].l.x}, y = {px[q].h.y, px[q].l.y};
+            const ff::FF<float> s = ff::add_accurate(x, y);
+            reinterpret_cast<float2 *>(red)[tid * 9 + q] = make_float2(s.h, s.l);
         }
-    } else {
-        if (PR == 2)
-#pragma unroll
-            for (int q = 0; q < 9; ++q)
-                acc[q] += (static_cast<double>(px[q].h.x) + static_cast<double>(px[q].l.x)) +
-                          (static_cast<double>(px[q].h.y) + static_cast<double>(px[q].l.y));
-        for (int o = span >> 1; o > 0; o >>= 1)
-#pragma unroll
-            for (int q = 0; q < 9; ++q)
-                acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
     }
-    if (L <= 32) {
-        if (valid && lane == 0)
+    __syncthreads();
+    // the lanes' sums (mixed: one per warp or group): S threads per value take
+    // every S-th lane, one adds their sums; four chains each (an FP64 addition
+    // waits about a hundred clocks for the one before)
+    const int stepl = PR == 1 ? (L < 32 ? L : 32) : 1, nl = L / stepl, nv = 9 * K;
+    const int S = max(1, min(T / nv, nl / 4));
+    auto lane_sum = [&](int v, int s0) {
+        const int k = v / 9, q = v - 9 * k;
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int e = s0; e < nl; e += 4 * S)
 #pragma unroll
-            for (int q = 0; q < 9; ++q)
-                part[g * 9 + q] = acc[q];
+            for (int c = 0; c < 4; ++c)
+                if (e + c * S < nl) {
+                    const int at = (k * L + (e + c * S) * stepl) * 9 + q;
+                    if (PR == 0) {
+                        s[c] += red[at];
+                    } else {
+                        const float2 w = reinterpret_cast<const float2 *>(red)[at];
+                        s[c] += to_double(w.x) + to_double(w.y);
+                    }
+                }
+        return (s[0] + s[1]) + (s[2] + s[3]);
+    };
+    if (S == 1) {
+        for (int u = tid; u < nv; u += T)
+            part[static_cast<size_t>(u) * pstride] = lane_sum(u, 0);
     } else {
-        if ((tid & 31) == 0)
-#pragma unroll
-            for (int q = 0; q < 9; ++q)
-                wred[w][q] = acc[q];
+        const double mine = tid < nv * S ? lane_sum(tid / S, tid % S) : 0.0;
         __syncthreads();
-        const int wpg = L >> 5;
-        if (tid < K)
+        red[tid] = mine;
+        __syncthreads();
+        if (tid < nv)
+            part[static_cast<size_t>(tid) * pstride] = sum4(red + tid * S, S);
+    }
+    if (PR == 2 && __syncthreads_or(spilled)) {
+        // long slices: the FP64 sums of the first iterations, added behind
+        __syncthreads();
 #pragma unroll
-            for (int q = 0; q < 9; ++q) {
-                double s = 0.0;
-                for (int u = 0; u < wpg; ++u)
-                    s += wred[tid * wpg + u][q];
-                part[tid * 9 + q] = s;
-            }
+        for (int q = 0; q < 9; ++q)
+            red[tid * 9 + q] = acc[q];
+        __syncthreads();
+        for (int u = tid; u < 9 * K; u += T) {
+            const int k = u / 9, q = u - 9 * k;
+            double s = part[static_cast<size_t>(u) * pstride];
+            for (int e = 0; e < L; ++e)
+                s += red[(k * L + e) * 9 + q];
+            part[static_cast<size_t>(u) * pstride] = s;
+        }
     }
     __syncthreads();
 }
 
-template <int PR>
-__global__ void __launch_bounds__(kStepThreads) step_kernel(StepArgs a)
+template <int PR, int T>
+__global__ void __launch_bounds__(T) step_kernel(StepArgs a)
 {
     cg::grid_group grid = cg::this_grid();
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ double red_d[32];
-    __shared__ int red_i[32];
+    __shared__ unsigned long long red_u[T / 32];
+    __shared__ int red_i[T / 32];
     __shared__ int s_act[kStepSmall];
-    __shared__ double s_iv[kStepSmall][9];
-    __shared__ double s_wred[kStepThreads / 32][9];
-    __shared__ double s_f[kStepSmall][9];
-    __shared__ int s_nb, s_qb[kStepSmall], s_blk[kStepSmall], s_cnt[kStepSmall];
-    const int B = gridDim.x, bk = blockIdx.x, tid = threadIdx.x, T = blockDim.x;
+    __shared__ __align__(8) unsigned char s_rec[kStepSmall * rows_of(PR) * word_of(PR)];
+    __shared__ double s_red[9 * T];  // sums of the lanes, then of the blocks
+    __shared__ CorrectScratch s_cor;
+    const int B = gridDim.x, bk = blockIdx.x, tid = threadIdx.x;
     const int per = (a.n + B - 1) / B;
     const int lo = min(a.n, bk * per), hi = min(a.n, lo + per);
     const int per_t = (hi - lo + T - 1) / T;
@@ -361,10 +408,10 @@ __global__ void __launch_bounds__(kStepThreads) step_kernel(StepArgs a)
     double last_t = 0.0;
     for (;;) {
         // schedule: this block's earliest t_i + dt_i, the particles reaching it
-        double mt = INFINITY;
+        unsigned long long mt = ~0ull;
         int ct = 0;
         for (int i = c0; i < c1; ++i) {
-            const double tt = a.t[i] + a.dt[i];
+            const unsigned long long tt = static_cast<unsigned long long>(__double_as_longlong(a.t[i] + a.dt[i]));
             if (tt < mt) {
                 mt = tt;
                 ct = 1;
@@ -372,14 +419,14 @@ __global__ void __launch_bounds__(kStepThreads) step_kernel(StepArgs a)
                 ++ct;
             }
         }
-        const double mb = block_min_d(mt, red_d);
-        const int mine = (mt == mb) ? ct : 0;
+        const unsigned long long mb = block_min_u64(mt, red_u);
+        const int mine = (mt == mb && mb != ~0ull) ? ct : 0;
         int tot_b = 0;
         const int ex = block_scan_excl(mine, red_i, &tot_b);
         if (mine > 0 && tot_b <= kStepSmall) {
             int pos = ex;
             for (int i = c0; i < c1; ++i)
-                if (a.t[i] + a.dt[i] == mb)
+                if (static_cast<unsigned long long>(__double_as_longlong(a.t[i] + a.dt[i])) == mb)
                     a.cand[bk * kStepSmall + pos++] = i;
         }
         if (tid == 0) {
@@ -387,17 +434,26 @@ __global__ void __launch_bounds__(kStepThreads) step_kernel(StepArgs a)
             a.bcnt[bk] = tot_b;
         }
         grid.sync();
-        // the same decision in every block
-        double mn = INFINITY;
-        for (int q = tid; q < B; q += T)
-            mn = fmin(mn, __ldcg(&a.bmin[q]));
-        mn = block_min_d(mn, red_d);
-        int c = 0;
-        for (int q = tid; q < B; q += T)
-            c += (__ldcg(&a.bmin[q]) == mn) ? __ldcg(&a.bcnt[q]) : 0;
-        int total = 0;
-        block_scan_excl(c, red_i, &total);
+        // the same decision in every block: thread tid looks at the blocks
+        // kQ tid .. kQ tid + kQ - 1
+        unsigned long long bm[kQ], mn_bits = ~0ull;
+        int bc[kQ];
+#pragma unroll
+        for (int e = 0; e < kQ; ++e) {
+            const int q = tid * kQ + e;
+            bm[e] = q < B ? __ldcg(&a.bmin[q]) : ~0ull;
+            bc[e] = q < B ? __ldcg(&a.bcnt[q]) : 0;
+            mn_bits = bm[e] < mn_bits ? bm[e] : mn_bits;
+        }
         const int err = *reinterpret_cast<volatile int *>(&a.ctl->err);
+        mn_bits = block_min_u64(mn_bits, red_u);
+        const double mn = __longlong_as_double(static_cast<long long>(mn_bits));
+        int c = 0;
+#pragma unroll
+        for (int e = 0; e < kQ; ++e)
+            c += bm[e] == mn_bits ? min(bc[e], kStepSmall + 1) : 0;
+        int total = 0;
+        int pos = block_scan_excl(c, red_i, &total);
         if (err) {
             reason = 2;
             break;
@@ -410,84 +466,68 @@ __global__ void __launch_bounds__(kStepThreads) step_kernel(StepArgs a)
             reason = 1;
             break;
         }
-        // the blocks holding the active set, in block order (at most total)
-        if (tid == 0)
-            s_nb = 0;
+        // active list, ascending: blocks in order, each block's list in order
+#pragma unroll
+        for (int e = 0; e < kQ; ++e)
+            if (bm[e] == mn_bits)
+                for (int u = 0; u < bc[e]; ++u)
+                    s_act[pos++] = (tid * kQ + e) * kStepSmall + u;
         __syncthreads();
-        for (int q = tid; q < B; q += T)
-            if (__ldcg(&a.bmin[q]) == mn && __ldcg(&a.bcnt[q]) > 0)
-                s_qb[atomicAdd(&s_nb, 1)] = q;
+        if (tid < total)
+            s_act[tid] = __ldcg(&a.cand[s_act[tid]]);
         __syncthreads();
-        const int nb = s_nb;
-        if (tid < nb) {
-            const int q = s_qb[tid];
-            int r = 0;
-            for (int u = 0; u < nb; ++u)
-                r += s_qb[u] < q ? 1 : 0;
-            s_blk[r] = q;
-            s_cnt[r] = __ldcg(&a.bcnt[q]);
-        }
-        __syncthreads();
-        // active list (ascending) and the predicted i-values
-        for (int k = tid; k < total; k += T) {
-            int base = 0, r = 0;
-            while (k >= base + s_cnt[r])
-                base += s_cnt[r++];
-            const int i = __ldcg(&a.cand[s_blk[r] * kStepSmall + (k - base)]);
-            s_act[k] = i;
-            ivalues<PR>(a, i, mn, s_iv[k]);
-        }
-        __syncthreads();
-        eval_slice<PR>(a, lo, hi, mn, total, s_iv, a.part + static_cast<size_t>(bk) * kStepSmall * 9, s_wred,
-                       smem);
+        eval_slice<PR, T>(a, lo, hi, mn, total, s_act, s_rec, a.part + bk, B, s_red, smem);
         grid.sync();
-        // owners: the partial sums of all blocks in block order, then correct
-        bool owns_any = false;
+        // this block's active particles (they are consecutive in the list)
+        int first_own = 0, own = 0;
         for (int k = 0; k < total; ++k) {
             const int i = s_act[k];
-            if (i < lo || i >= hi)
-                continue;
-            owns_any = true;
-            double s9[9];
-#pragma unroll
-            for (int q = 0; q < 9; ++q)
-                s9[q] = 0.0;
-            for (int q2 = tid; q2 < B; q2 += T) {
-                const double *pp = a.part + (static_cast<size_t>(q2) * kStepSmall + k) * 9;
-#pragma unroll
-                for (int q = 0; q < 9; ++q)
-                    s9[q] += __ldcg(&pp[q]);
-            }
-            // fixed-order combination of the threads' sums
-            for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                for (int q = 0; q < 9; ++q)
-                    s9[q] += __shfl_xor_sync(0xffffffffu, s9[q], o);
-            if ((tid & 31) == 0)
-#pragma unroll
-                for (int q = 0; q < 9; ++q)
-                    s_wred[tid >> 5][q] = s9[q];
-            __syncthreads();
-            if (tid < 9) {
-                double s = 0.0;
-                for (int u = 0; u < (T >> 5); ++u)
-                    s += s_wred[u][tid];
-                s_f[k][tid] = s;
-            }
-            __syncthreads();
+            if (i < lo)
+                first_own = k + 1;
+            else if (i < hi)
+                ++own;
         }
-        if (owns_any)
-            for (int k = tid; k < total; k += T) {
-                const int i = s_act[k];
-                if (i < lo || i >= hi)
-                    continue;
-                double f[9];
+        for (int o0 = 0; o0 < own; o0 += 32) {
+            const int no = min(32, own - o0);
+            // the partial sums of all blocks: S threads per value take every
+            // S-th block, one adds their sums in order
+            const int nv = 9 * no;
+            const int S = nv <= T ? T / nv : 1;
+            for (int u = tid; u < nv * S; u += T) {
+                const int v = u / S, s = u - v * S;
+                const double *pp = a.part + (static_cast<size_t>(first_own + o0) * 9 + v) * B;
+                double sum[4] = {0.0, 0.0, 0.0, 0.0};
+                constexpr int U = 12;  // loads in flight
+                for (int q = s; q < B; q += U * S) {
+                    double w[U];
 #pragma unroll
-                for (int q = 0; q < 9; ++q)
-                    f[q] = s_f[k][q];
-                correct_particle_fp64(a.st, a.t, a.dt, static_cast<size_t>(a.n), i, mn, f, a.eta, a.dt_min,
-                                      a.dt_max, a.dt_shared, a.ctl, a.noise);
+                    for (int e = 0; e < U; ++e)
+                        w[e] = q + e * S < B ? __ldcg(pp + q + e * S) : 0.0;
+#pragma unroll
+                    for (int e = 0; e < U; ++e)
+                        if (q + e * S < B)
+                            sum[e & 3] += w[e];
+                }
+                s_red[u] = (sum[0] + sum[1]) + (sum[2] + sum[3]);
             }
+            __syncthreads();
+            if (S > 1) {
+                const double sum = tid < nv ? sum4(s_red + tid * S, S) : 0.0;
+                __syncthreads();
+                if (tid < nv)
+                    s_red[tid] = sum;
+                __syncthreads();
+            }
+            const int lane = tid & 31, d = tid >> 5;
+            const bool valid = d < 3 && lane < no;
+            double f[3] = {0.0, 0.0, 0.0};
+            if (valid)
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    f[q] = s_red[lane * 9 + 3 * q + d];
+            correct_group_fp64(a.st, a.t, a.dt, static_cast<size_t>(a.n), valid ? s_act[first_own + o0 + lane] : 0,
+                               valid, mn, f, a.eta, a.dt_min, a.dt_max, a.dt_shared, a.ctl, a.noise, s_cor);
+        }
         if (bk == 0) {
             for (int k = tid; k < total; k += T)
                 a.act[k] = s_act[k];
@@ -514,25 +554,29 @@ __global__ void __launch_bounds__(kStepThreads) step_kernel(StepArgs a)
     }
 }
 
-template <int PR>
-cudaError_t launch_stepper(nb_ctx *c, StepArgs &a, int grid_max)
+template <int PR, int T>
+cudaError_t launch_stepper(nb_ctx *c, StepArgs &a, int grid)
 {
     const size_t smem = static_cast<size_t>(kChunkCap) * rec_bytes(PR);
-    cudaError_t e = cudaFuncSetAttribute(step_kernel<PR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(step_kernel<PR, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem));
     if (e != cudaSuccess)
         return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_kernel<PR>, kStepThreads, smem);
-    if (e != cudaSuccess)
-        return e;
-    if (per_sm < 1)
-        return cudaErrorInvalidConfiguration;
-    int grid = std::min(c->sm_count * per_sm, grid_max);                  // all blocks resident
-    grid = std::min(grid, std::max(1, static_cast<int>((c->n + 31) / 32)));  // >= 32 particles per block
     void *args[] = {&a};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(step_kernel<PR>), dim3(grid),
-                                       dim3(kStepThreads), args, smem, c->stream);
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(step_kernel<PR, T>), dim3(grid), dim3(T), args,
+                                       smem, c->stream);
+}
+
+// One block per SM (with two, every barrier and sum over blocks grows: EX
+// N = 8192 28.2 us a step), all of them resident.
+template <int PR>
+cudaError_t launch_stepper(nb_ctx *c, StepArgs &a, int grid_max)
+{
+    const int slice = PR == 0 ? kSliceFp64 : kSliceFp32;
+    const int grid = std::min({c->sm_count, grid_max, kQ * 128,
+                               std::max(1, static_cast<int>((c->n + slice - 1) / slice))});
+    return c->n >= static_cast<int64_t>(grid) * kSliceWide ? launch_stepper<PR, 256>(c, a, grid)
+                                                           : launch_stepper<PR, 128>(c, a, grid);
 }
 
 }  // namespace
@@ -572,7 +616,7 @@ cudaError_t nb_run_stepper(nb_ctx *c, double t_end, int64_t log_cap, int64_t log
     a.dt_shared = c->cfg.dt_shared;
     a.t_end = t_end;
     a.drop_lo = c->cfg.precision == NB_SP ? 1 : 0;
-    a.bmin = c->stp_bmin;
+    a.bmin = reinterpret_cast<unsigned long long *>(c->stp_bmin);
     a.bcnt = c->stp_bcnt;
     a.cand = c->stp_cand;
     a.part = c->stp_part;

@@ -118,14 +118,29 @@ nb_status sync_ctl(nb_ctx *c)
 
 // The complete active set 0 .. n-1 against all particles, each unordered pair
 // once (k_sym.cu), where the context's plan for it is estimated faster than the
-// ordinary kernels and no launch shape is asked for.  *done says whether it
-// ran.
+// ordinary kernels and no launch shape is asked for.  Its workspace is
+// allocated by the first such evaluation and kept.  *done says whether it ran:
+// not where the workspace cannot be had (no memory, or a stream that is being
+// captured before an evaluation outside of a capture).
 nb_status eval_all_pairs(nb_ctx *c, double *out, bool *done)
 {
     *done = false;
     const nb_tiles &t = c->cfg.tiles;
     if (!c->sym_use || c->inject || t.ki || t.threads || t.jtile || t.lanes || t.split || t.junroll)
         return NB_OK;
+    if (!c->sym_work) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+            (void)cudaGetLastError();
+            return NB_OK;
+        }
+        if (cudaMalloc(&c->sym_work, c->sym_plan.bytes) != cudaSuccess) {
+            (void)cudaGetLastError();
+            c->sym_work = nullptr;
+            c->sym_use = false;  // the memory is the caller's to use: not tried again
+            return NB_OK;
+        }
+    }
     const bool rows = nb_jrows(c->cfg.precision) > 0;
     int launches = 0;
     CU(c, nb_launch_sym(c->cfg.precision, c->sym_plan, rows ? static_cast<const void *>(c->jf32) : c->jb64,
@@ -431,13 +446,6 @@ nb_status nb_init(nb_ctx **out, int64_t n, const double *m, const double *x, con
         (void)nb_auto_tiles(c, n, nb_tiles{}, 0, &us);
         c->sym_plan = nb_sym_plan(cf.precision, n, c->sm_count);
         c->sym_use = c->sym_plan.us < us;
-        // its workspace, so that no evaluation allocates; without the memory
-        // the ordinary kernels run
-        if (c->sym_use && cudaMalloc(&c->sym_work, c->sym_plan.bytes) != cudaSuccess) {
-            (void)cudaGetLastError();
-            c->sym_work = nullptr;
-            c->sym_use = false;
-        }
     }
     if (const int rows = nb_jrows(cf.precision)) {
         CUI(cudaMalloc(&c->jf32, rows * static_cast<size_t>(c->npad) * sizeof(float)));

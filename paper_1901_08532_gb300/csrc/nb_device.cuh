@@ -149,12 +149,53 @@ __device__ __forceinline__ Taylor taylor(double x, double v, double a, double j,
     return r;
 }
 
+// -------------------------------------------- FP64 <-> FP32 on the integer pipe
+
+// Conversion instructions between FP64 and FP32 run at the FP64 pipe's rate
+// (1/64 of FP32 on GB300), a few integer instructions at a quarter of it and
+// beside it: predict_kernel of 2^20 particles, mixed 119 -> 92 us, EX 162 -> 121 us.
+
+// x rounded to the nearest FP32 value (ties to even), as __double2float_rn.
+__device__ __forceinline__ float to_float(double x)
+{
+    const unsigned hi = static_cast<unsigned>(__double2hiint(x)), lo = static_cast<unsigned>(__double2loint(x));
+    // biased exponents 897 .. 1149 stay normal in FP32 after rounding
+    if (((hi >> 20) & 0x7ff) - 897u > 252u)
+        return ((hi & 0x7fffffffu) | lo) == 0 ? __uint_as_float(hi) : __double2float_rn(x);
+    // exponent re-biased, mantissa cut to 23 bits; the 29 bits dropped decide
+    const unsigned kept = ((hi & 0x7fffffffu) - (896u << 20)) << 3 | lo >> 29;
+    const unsigned rest = lo << 3;  // dropped bits, left-aligned
+    const unsigned up = rest > 0x80000000u || (rest == 0x80000000u && (kept & 1)) ? 1u : 0u;
+    return __uint_as_float((hi & 0x80000000u) | (kept + up));
+}
+
+// x as a double (exact).
+__device__ __forceinline__ double to_double(float x)
+{
+    const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+    if (m != 0 && (m >> 23) - 1u > 253u)
+        return static_cast<double>(x);  // subnormal, infinite, NaN
+    return __hiloint2double(static_cast<int>((u & 0x80000000u) | (m == 0 ? 0u : (m >> 3) + (896u << 20))),
+                            static_cast<int>(u << 29));
+}
+
 // ------------------------------------------------------- step quantisation
 
 // Largest power of two <= x for positive normal x (clears the mantissa).
 __device__ __forceinline__ double pow2_floor(double x)
 {
     return __hiloint2double(__double2hiint(x) & 0x7ff00000, 0);
+}
+
+// 1/h, by the exponent alone where h is a power of two (exact either way; an
+// FP64 division is a chain of about ten FP64-pipe instructions).
+__device__ __forceinline__ double inverse_step(double h)
+{
+    const int hi = __double2hiint(h);
+    const unsigned e = static_cast<unsigned>(hi) >> 20;
+    if ((hi & 0xfffff) == 0 && __double2loint(h) == 0 && e >= 1 && e <= 2045)
+        return __hiloint2double(static_cast<int>((2046 - e) << 20), 0);
+    return 1.0 / h;
 }
 
 __device__ __forceinline__ double quantise(double crit, double dt_old, double t1, double dt_min, double dt_max,
@@ -170,7 +211,7 @@ __device__ __forceinline__ double quantise(double crit, double dt_old, double t1
     }
     if (dt_old > 0.0 && p > dt_old) {
         const double d2 = 2.0 * dt_old;
-        const double q = t1 * (1.0 / d2);  // exact: d2 is a power of two
+        const double q = t1 * inverse_step(d2);  // exact: d2 is a power of two
         p = (q == trunc(q)) ? d2 : dt_old;
     }
     return p;
@@ -221,6 +262,60 @@ __device__ __forceinline__ double aarseth_dt(const double (&n2)[6], double eta)
     if (A1 == 0.0 && A4 == 0.0)
         return INFINITY;
     return eta * cbrt(A1 / A4);
+}
+
+// log2 of a positive normal x as an integer and a fraction in [0, 1).
+struct Log2 {
+    int e;
+    float f;
+};
+__device__ __forceinline__ bool log2_of(double x, Log2 &r)
+{
+    const unsigned hi = static_cast<unsigned>(__double2hiint(x));
+    if ((hi >> 20) - 1u > 2045u)
+        return false;  // zero, negative, subnormal, infinite, NaN
+    r.e = static_cast<int>(hi >> 20) - 1023;
+    r.f = __log2f(__uint_as_float(0x3f800000u | (hi & 0xfffffu) << 3 | static_cast<unsigned>(__double2loint(x)) >> 29));
+    return true;
+}
+
+// floor(log2(aarseth_dt(n2, eta))) in FP32, where that is beyond doubt: *k is
+// set and true returned unless the logarithm lies within 4e-5 of an integer or
+// a norm is zero or not finite, where the caller takes aarseth_dt.  The
+// step is used rounded down to a power of two, so the decision is the same as
+// with FP64 roots (eight square roots, a division and a cube root: about 70
+// FP64-pipe instructions in a chain).  Exponents stay integers (in units of
+// 1/12), so each logarithm's fraction is below 13 and its rounding and that
+// of __log2f and exp2f (2^-22 each) sum to less than 1e-5.
+__device__ __forceinline__ bool aarseth_log2(const double (&n2)[6], double eta, int *k)
+{
+    Log2 l[6], le;
+    bool ok = log2_of(eta, le);
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+        ok = log2_of(n2[q], l[q]) && ok;
+    if (!ok)
+        return false;
+    // log2 A = log2(2^x + 2^y), x = (l0 + l2) / 4, y = l1 / 2
+    int ae[2];
+    float af[2];
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+        const int xe = l[3 * g].e + l[3 * g + 2].e, ye = 2 * l[3 * g + 1].e;  // in units of 1/4
+        const float xf = 0.25f * (l[3 * g].f + l[3 * g + 2].f), yf = 0.5f * l[3 * g + 1].f;
+        const float d = 0.25f * static_cast<float>(xe - ye) + (xf - yf);
+        const bool big = d >= 0.0f;
+        ae[g] = big ? xe : ye;
+        af[g] = (big ? xf : yf) + __log2f(1.0f + exp2f(-fabsf(d)));
+    }
+    // log2 eta + (log2 A1 - log2 A4) / 3, in units of 1/12 and a fraction
+    const int e12 = ae[0] - ae[1] + 12 * le.e;
+    const float f = le.f + (af[0] - af[1]) * (1.0f / 3.0f);
+    const int e = e12 >= 0 ? e12 / 12 : -((11 - e12) / 12);  // floor
+    const float r = f + static_cast<float>(e12 - 12 * e) * (1.0f / 12.0f);
+    const float fl = floorf(r), fr = r - fl;
+    *k = e + static_cast<int>(fl);
+    return fr > 4e-5f && fr < 1.0f - 4e-5f && *k > -1000 && *k < 1000;
 }
 
 // Starting step eta_s min(|a|/|j|, sqrt(|a|/|s|)) from |a| and the squared

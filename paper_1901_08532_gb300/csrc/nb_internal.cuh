@@ -52,8 +52,10 @@ struct SymPlan {
     size_t ns = 0, pi_slots = 0, bytes = 0;
 };
 // Bytes of partial sums that a plan may use where it needs more than the two
-// slots (72 B per particle each) of the smallest one.
-constexpr double kSymSlotBytes = 1e9;
+// slots (72 B per particle each) of the smallest one: 24 slots, at least
+// 512 MB, at most 1 GB (65536 particles mixed 4.83 ms, with 256 MB 5.05 ms; 2 GB
+// would gain 1 % from 131072 particles).
+constexpr double kSymSlotBytes = 1e9, kSymMinBytes = 512e6, kSymSlots = 24.0;
 
 struct nb_ctx {
     int dev = 0;
