@@ -39,6 +39,7 @@
 #include <string>
 #include <vector>
 
+#include "nb_block.cuh"
 #include "nb_correct.cuh"
 #include "nb_device.cuh"
 #include "nb_ff.cuh"
@@ -118,44 +119,6 @@ struct EnsArgs {
 constexpr int kEnsThreads = 256;
 constexpr int kMaxCluster = 16;  // blocks per system: 8 portable, 16 with the opt-in attribute
 
-__device__ __forceinline__ double block_min(double v, double *red)
-{
-    for (int o = 16; o > 0; o >>= 1)
-        v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
-    const int w = threadIdx.x >> 5;
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0)
-        red[w] = v;
-    __syncthreads();
-    double r = red[0];
-    for (int q = 1; q < static_cast<int>(blockDim.x >> 5); ++q)
-        r = fmin(r, red[q]);
-    return r;
-}
-
-__device__ int block_exclusive_scan(int v, int *red, int *total)
-{
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int incl = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o)
-            incl += u;
-    }
-    __syncthreads();
-    if (lane == 31)
-        red[w] = incl;
-    __syncthreads();
-    int base = 0, tot = 0;
-    for (int q = 0; q < nw; ++q) {
-        if (q < w)
-            base += red[q];
-        tot += red[q];
-    }
-    *total = tot;
-    return base + incl - v;
-}
-
 // Taylor prediction of particle i to tp (FP64, through crackle).
 __device__ __forceinline__ void predict_one(const EnsArgs &a, int i, double tp, Taylor (&p)[3])
 {
@@ -215,11 +178,11 @@ __device__ __forceinline__ void predict_one_mixed(const EnsArgs &a, int i, doubl
 __device__ __forceinline__ void store_xv32(const EnsArgs &a, int i, int k, double x, double v)
 {
     const size_t P = static_cast<size_t>(a.P);
-    const float xh = __double2float_rn(x), vh = __double2float_rn(v);
+    const float xh = to_float(x), vh = to_float(v);
     a.st32[(15 + k) * P + i] = xh;
-    a.st32[(18 + k) * P + i] = __double2float_rn(x - static_cast<double>(xh));
+    a.st32[(18 + k) * P + i] = to_float(x - to_double(xh));
     a.st32[k * P + i] = vh;
-    a.st32[(21 + k) * P + i] = __double2float_rn(v - static_cast<double>(vh));
+    a.st32[(21 + k) * P + i] = to_float(v - to_double(vh));
 }
 
 // The mixed j-record of particle i predicted to tp.  NB_MIXED (PR 1): the
@@ -237,11 +200,11 @@ __device__ __forceinline__ void mixed_record(const EnsArgs &a, int i, double tp,
     predict_one(a, i, tp, p);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const float h = __double2float_rn(p[k].x);
+        const float h = to_float(p[k].x);
         r.xh[k] = h;
-        r.xl[k] = __double2float_rn(p[k].x - static_cast<double>(h));
-        r.v[k] = __double2float_rn(p[k].v);
-        r.a[k] = __double2float_rn(p[k].a);
+        r.xl[k] = to_float(p[k].x - to_double(h));
+        r.v[k] = to_float(p[k].v);
+        r.a[k] = to_float(p[k].a);
     }
 }
 
@@ -261,7 +224,7 @@ __device__ void predict_slice(const EnsArgs &a, int lo, int hi, double tp)
                 a.jf32[(7 + k) * P + i] = r.v[k];
                 a.jf32[(10 + k) * P + i] = r.a[k];
             }
-            a.jf32[3 * P + i] = __double2float_rn(a.m[i]);
+            a.jf32[3 * P + i] = to_float(a.m[i]);
         } else if (EXP) {
             // 20 FP32 rows: hi then lo of x, v, a (three rows each), m hi, m lo
             Taylor p[3];
@@ -271,14 +234,14 @@ __device__ void predict_slice(const EnsArgs &a, int lo, int hi, double tp)
                 const double q[3] = {p[k].x, p[k].v, p[k].a};
 #pragma unroll
                 for (int g = 0; g < 3; ++g) {
-                    const float h = __double2float_rn(q[g]);
+                    const float h = to_float(q[g]);
                     a.jf32[(6 * g + k) * P + i] = h;
-                    a.jf32[(6 * g + 3 + k) * P + i] = __double2float_rn(q[g] - static_cast<double>(h));
+                    a.jf32[(6 * g + 3 + k) * P + i] = to_float(q[g] - to_double(h));
                 }
             }
-            const float mh = __double2float_rn(a.m[i]);
+            const float mh = to_float(a.m[i]);
             a.jf32[18 * P + i] = mh;
-            a.jf32[19 * P + i] = __double2float_rn(a.m[i] - static_cast<double>(mh));
+            a.jf32[19 * P + i] = to_float(a.m[i] - to_double(mh));
         } else {
             Taylor p[3];
             predict_one(a, i, tp, p);
@@ -604,267 +567,74 @@ __device__ __forceinline__ void correct_particle(const EnsArgs &a, int i, double
 // blocks per SM); its steps with more active particles take the j-split
 // large-set path, which is as well balanced.
 constexpr int kSmallMax = 128;
+// Sums of 32 particles, or of 256 threads, ahead of a corrector's scratch.
+constexpr size_t kSumBytes = 32 * 9 * sizeof(double);
 __host__ __device__ constexpr int small_set(int pr) { return pr == 1 || pr == 3 ? 16 : kSmallMax; }
 
-// i-values of the small active set: FP64 x, v, a; in mixed precision the
-// same slots hold 12 negated FP32 values (x_hi, x_lo, v, a) of the record the
-// predictor writes for particle i.
-template <int PR>
-__device__ __forceinline__ void store_ivalues(const EnsArgs &a, int i, double tn, double *iv)
-{
-    [[maybe_unused]] constexpr bool MIXED = PR == 1 || PR == 3, EXP = PR == 2;
-    if (MIXED) {
+// The predicted record of NB_MIXED32 as eval_slice's Record (FP32 prediction,
+// not worth spreading by component: component 0 writes it all).
+struct Mixed32Record {
+    const EnsArgs &a;
+    double tn;
+    __device__ __forceinline__ void operator()(int i, int d, void *rows, int stride) const
+    {
+        if (d > 0)
+            return;
         MixedRec r;
-        mixed_record<PR>(a, i, tn, r);
-        float *f = reinterpret_cast<float *>(iv);
+        predict_one_mixed(a, i, tn, r);
+        float *f = static_cast<float *>(rows);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            f[k] = -r.xh[k];
-            f[3 + k] = -r.xl[k];
-            f[6 + k] = -r.v[k];
-            f[9 + k] = -r.a[k];
+            f[k * stride] = r.xh[k];
+            f[(4 + k) * stride] = r.xl[k];
+            f[(7 + k) * stride] = r.v[k];
+            f[(10 + k) * stride] = r.a[k];
         }
-    } else if (EXP) {
-        // 18 negated FP32 values: hi then lo of x, v, a (the j-record's split)
-        Taylor p[3];
-        predict_one(a, i, tn, p);
-        float *f = reinterpret_cast<float *>(iv);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const double q[3] = {p[k].x, p[k].v, p[k].a};
-#pragma unroll
-            for (int g = 0; g < 3; ++g) {
-                const float h = __double2float_rn(q[g]);
-                f[6 * g + k] = -h;
-                f[6 * g + 3 + k] = -__double2float_rn(q[g] - static_cast<double>(h));
-            }
-        }
-    } else {
-        Taylor p[3];
-        predict_one(a, i, tn, p);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            iv[k] = p[k].x;
-            iv[3 + k] = p[k].v;
-            iv[6 + k] = p[k].a;
-        }
+        f[3 * stride] = to_float(a.m[i]);
     }
+};
+
+// Partial sums of the K active particles over this block's slice, part[K][9].
+template <int PR>
+__device__ __forceinline__ void eval_small(const EnsArgs &a, int lo, int hi, double tn, int K, const int *act,
+                                           void *rec, int kmax, double *part, unsigned char *smem)
+{
+    constexpr int AR = PR == 3 ? 1 : PR;  // the pair arithmetic
+    double *red = reinterpret_cast<double *>(smem);  // the chunk is done with when the sums meet
+    auto run = [&](const auto &record) {
+        eval_slice<AR>(record, a.eps2, lo, hi, K, act, rec, kmax, part, 1, red, smem, 2 * a.jtile, blockDim.x);
+    };
+    if constexpr (PR == 3)
+        run(Mixed32Record{a, tn});
+    else
+        run(PredictedRecord<AR>{{a.st, a.t, a.m, static_cast<size_t>(a.P), 0}, tn});
 }
 
-// Partial sums of the K active particles (i-values in iv) over the j of
-// [lo, hi), written to part[K][9].  The j are predicted to tn chunk by chunk
-// straight into shared memory (cap records per chunk, the layout of the
-// evaluation buffer: 13 or 20 FP32 rows, or 5 rows of double2), so the sums read
-// on-chip data only.  L = T / K2 lanes per active particle (K2 the power of
-// two >= K); lanes take every L-th j (pair of j in mixed precision) and are
-// combined in a fixed order.
+// Corrects the active particles list[0 .. no) (no <= 32) from the sums f9 of
+// `no` particles ([no][9], shared memory); scratch: a CorrectScratch.
 template <int PR>
-__device__ void eval_small(const EnsArgs &a, int lo, int hi, double tn, int K, const double (*iv)[9],
-                           double (*part)[9], double (*wred)[9], unsigned char *smem, int cap)
+__device__ __forceinline__ void correct_few(const EnsArgs &a, const int *list, int no, double tn, const double *f9,
+                                            CorrectScratch &scratch)
 {
-    [[maybe_unused]] constexpr bool MIXED = PR == 1 || PR == 3, EXP = PR == 2;
-    const int T = blockDim.x, tid = threadIdx.x;
-    int K2 = 1;
-    while (K2 < K)
-        K2 <<= 1;
-    const int L = T / K2;
-    const int g = tid / L, lane = tid - g * L;
-    const bool valid = g < K;
-    const int gi = valid ? g : 0;
-    double acc[9];
-#pragma unroll
-    for (int q = 0; q < 9; ++q)
-        acc[q] = 0.0;
-    float2 ni[12];
-    float2 pt[9];
-    float ah[9], al[9];  // mixed: compensated (hi, lo) running sums
-#pragma unroll
-    for (int q = 0; q < 9; ++q)
-        ah[q] = al[q] = 0.0f;
-    int cnt = 0;
-    ExI<float2> nie;
-    ff::FF<float2> px[9];
-    if (EXP) {
-        const float *ivf = reinterpret_cast<const float *>(iv[gi]);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            nie.x[k] = {f2(ivf[k]), f2(ivf[3 + k])};
-            nie.v[k] = {f2(ivf[6 + k]), f2(ivf[9 + k])};
-            nie.a[k] = {f2(ivf[12 + k]), f2(ivf[15 + k])};
-        }
-#pragma unroll
-        for (int q = 0; q < 9; ++q)
-            px[q] = {f2(0.0f), f2(0.0f)};
-    }
-    if (MIXED) {
-        const float *ivf = reinterpret_cast<const float *>(iv[gi]);
-#pragma unroll
-        for (int q = 0; q < 12; ++q)
-            ni[q] = f2(ivf[q]);
-#pragma unroll
-        for (int q = 0; q < 9; ++q)
-            pt[q] = f2(0.0f);
-    }
-    const float2 eps2f = f2(static_cast<float>(a.eps2));
-    float *sf = reinterpret_cast<float *>(smem);
-    double2 *sd = reinterpret_cast<double2 *>(smem);
-    for (int b = lo; b < hi; b += cap) {
-        const int len = min(cap, hi - b);
-        for (int u = tid; u < len; u += T) {
-            const double mj = a.m[b + u];
-            if (MIXED) {
-                MixedRec r;
-                mixed_record<PR>(a, b + u, tn, r);
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    sf[k * cap + u] = r.xh[k];
-                    sf[(4 + k) * cap + u] = r.xl[k];
-                    sf[(7 + k) * cap + u] = r.v[k];
-                    sf[(10 + k) * cap + u] = r.a[k];
-                }
-                sf[3 * cap + u] = __double2float_rn(mj);
-            } else if (EXP) {
-                Taylor p[3];
-                predict_one(a, b + u, tn, p);
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const double q[3] = {p[k].x, p[k].v, p[k].a};
-#pragma unroll
-                    for (int gg = 0; gg < 3; ++gg) {
-                        const float h = __double2float_rn(q[gg]);
-                        sf[(6 * gg + k) * cap + u] = h;
-                        sf[(6 * gg + 3 + k) * cap + u] = __double2float_rn(q[gg] - static_cast<double>(h));
-                    }
-                }
-                const float mh = __double2float_rn(mj);
-                sf[18 * cap + u] = mh;
-                sf[19 * cap + u] = __double2float_rn(mj - static_cast<double>(mh));
-            } else {
-                Taylor p[3];
-                predict_one(a, b + u, tn, p);
-                sd[u] = make_double2(p[0].x, p[1].x);
-                sd[cap + u] = make_double2(p[2].x, mj);
-                sd[2 * cap + u] = make_double2(p[0].v, p[1].v);
-                sd[3 * cap + u] = make_double2(p[2].v, p[0].a);
-                sd[4 * cap + u] = make_double2(p[1].a, p[2].a);
-            }
-        }
-        __syncthreads();
-        if (EXP) {
-            const float e2h = __double2float_rn(a.eps2);
-            const ff::FF<float2> eps2x = {f2(e2h), f2(__double2float_rn(a.eps2 - static_cast<double>(e2h)))};
-            for (int jj = 2 * lane; jj < len; jj += 2 * L) {
-                float2 c[NCX];
-                if (jj + 1 < len) {
-#pragma unroll
-                    for (int r = 0; r < NCX; ++r)
-                        c[r] = *reinterpret_cast<const float2 *>(sf + r * cap + jj);
-                } else {
-                    // odd tail: the second half repeats the first j with no mass
-#pragma unroll
-                    for (int r = 0; r < NCX; ++r) {
-                        const float x0 = sf[r * cap + jj];
-                        c[r] = make_float2(x0, r >= 18 ? 0.0f : x0);
-                    }
-                }
-                pair_ex(c, nie, eps2x, px);
-                if (++cnt == 32) {
-#pragma unroll
-                    for (int q = 0; q < 9; ++q) {
-                        acc[q] += (static_cast<double>(px[q].h.x) + static_cast<double>(px[q].l.x)) +
-                                  (static_cast<double>(px[q].h.y) + static_cast<double>(px[q].l.y));
-                        px[q] = {f2(0.0f), f2(0.0f)};
-                    }
-                    cnt = 0;
-                }
-            }
-        } else if (MIXED) {
-            for (int jj = 2 * lane; jj < len; jj += 2 * L) {
-                float2 c[NCF];
-                if (jj + 1 < len) {
-#pragma unroll
-                    for (int r = 0; r < NCF; ++r)
-                        c[r] = *reinterpret_cast<const float2 *>(sf + r * cap + jj);
-                } else {
-                    // odd tail: the second half repeats the first j with no mass
-#pragma unroll
-                    for (int r = 0; r < NCF; ++r) {
-                        const float x0 = sf[r * cap + jj];
-                        c[r] = make_float2(x0, r == 3 ? 0.0f : x0);
-                    }
-                }
-                pair_mixed2(c, ni, eps2f, pt);
-                if (++cnt == 32) {
-#pragma unroll
-                    for (int q = 0; q < 9; ++q) {
-                        two_sum_acc(ah[q], al[q], __fadd_rn(pt[q].x, pt[q].y));
-                        pt[q] = f2(0.0f);
-                    }
-                    cnt = 0;
-                }
-            }
-        } else {
-            const double *v = iv[gi];
-            for (int jj = lane; jj < len; jj += L)
-                pair_fp64(sd[jj], sd[cap + jj], sd[2 * cap + jj], sd[3 * cap + jj], sd[4 * cap + jj], v[0],
-                          v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8], a.eps2, acc);
-        }
-        __syncthreads();
-    }
-    const int w = tid >> 5;
-    const int span = L < 32 ? L : 32;  // lanes combined by shuffles
-    if (EXP)
-#pragma unroll
-        for (int q = 0; q < 9; ++q)
-            acc[q] += (static_cast<double>(px[q].h.x) + static_cast<double>(px[q].l.x)) +
-                      (static_cast<double>(px[q].h.y) + static_cast<double>(px[q].l.y));
-    if (MIXED) {
-        // fixed-order double-word sums across the lanes; one FP64 conversion
-        // per group (or warp) leader
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            two_sum_acc(ah[q], al[q], __fadd_rn(pt[q].x, pt[q].y));
-            for (int o = span >> 1; o > 0; o >>= 1) {
-                const float oh = __shfl_xor_sync(0xffffffffu, ah[q], o);
-                const float ol = __shfl_xor_sync(0xffffffffu, al[q], o);
-                two_sum_acc(ah[q], al[q], oh);
-                al[q] = __fadd_rn(al[q], ol);
-            }
-        }
-        if ((tid & (span - 1)) == 0)
+    const int tid = threadIdx.x, lane = tid & 31, d = tid >> 5;
+    if (PR == 3 || blockDim.x < 96) {
+        if (tid < no) {
+            double f[9];
 #pragma unroll
             for (int q = 0; q < 9; ++q)
-                acc[q] = static_cast<double>(ah[q]) + static_cast<double>(al[q]);
-    } else {
-        for (int o = span >> 1; o > 0; o >>= 1)
-#pragma unroll
-            for (int q = 0; q < 9; ++q)
-                acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+                f[q] = f9[tid * 9 + q];
+            correct_particle<PR>(a, list[tid], tn, f);
+        }
+        return;
     }
-    if (L <= 32) {
-        if (valid && lane == 0)
+    const bool valid = d < 3 && lane < no;
+    double f[3] = {0.0, 0.0, 0.0};
+    if (valid)
 #pragma unroll
-            for (int q = 0; q < 9; ++q)
-                part[g][q] = acc[q];
-    } else {
-        if ((tid & 31) == 0)
-#pragma unroll
-            for (int q = 0; q < 9; ++q)
-                wred[w][q] = acc[q];
-        __syncthreads();
-        const int wpg = L >> 5;
-        if (tid < K)
-#pragma unroll
-            for (int q = 0; q < 9; ++q) {
-                double sum = 0.0;
-                for (int u = 0; u < wpg; ++u)
-                    sum += wred[tid * wpg + u][q];
-                part[tid][q] = sum;
-            }
-    }
-    // the chunk area is also a TMA destination in later steps
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
+        for (int q = 0; q < 3; ++q)
+            f[q] = f9[lane * 9 + 3 * q + d];
+    correct_group_fp64(a.st, a.t, a.dt, static_cast<size_t>(a.P), valid ? list[lane] : 0, valid, tn, f, a.eta, a.dt_min,
+                       a.dt_max, a.dt_shared, a.ctl, a.noise, scratch);
 }
 
 // Start-up stores for slots [s0, s1) (all particles, in order).
@@ -943,19 +713,19 @@ __global__ void __launch_bounds__(kEnsThreads, 1) ensemble_kernel(EnsArgs a)
     [[maybe_unused]] constexpr bool MIXED = PR == 1 || PR == 3, EXP = PR == 2;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar[2];
-    __shared__ double red_d[32];
+    __shared__ unsigned long long red_u[32];
     __shared__ int red_i[32];
     __shared__ int s_job;
     __shared__ int s_fail;
-    __shared__ double s_min2[2];
+    __shared__ unsigned long long s_min2[2];
     __shared__ int s_cnt2[2];
     constexpr int KS = small_set(PR);
     __shared__ int s_cand[2][KS];
     __shared__ int s_act[KS];
     __shared__ int s_rcnt[kMaxCluster];
-    __shared__ double s_iv[KS][9];
-    __shared__ double s_part[KS][9];
-    __shared__ double s_wred[kEnsThreads / 32][9];
+    constexpr int AR = PR == 3 ? 1 : PR;
+    __shared__ __align__(8) unsigned char s_rec[KS * rows_of(AR) * word_of(AR)];
+    __shared__ double s_part[KS * 9];
     __shared__ long long s_log_ip;
     cg::cluster_group cl = cg::this_cluster();
     const int rank = static_cast<int>(cl.block_rank());
@@ -1012,10 +782,11 @@ __global__ void __launch_bounds__(kEnsThreads, 1) ensemble_kernel(EnsArgs a)
             const int par = static_cast<int>(steps & 1);
             // schedule, one pass: the slice's earliest t_i + dt_i and how many
             // particles reach it; a small set is listed in shared memory
-            double mt = INFINITY;
+            unsigned long long mt = ~0ull;
             int ct = 0;
             for (int i = c0; i < c1; ++i) {
-                const double tt = a.t[i] + a.dt[i];
+                const unsigned long long tt =
+                    static_cast<unsigned long long>(__double_as_longlong(a.t[i] + a.dt[i]));
                 if (tt < mt) {
                     mt = tt;
                     ct = 1;
@@ -1023,15 +794,15 @@ __global__ void __launch_bounds__(kEnsThreads, 1) ensemble_kernel(EnsArgs a)
                     ++ct;
                 }
             }
-            const double mb = block_min(mt, red_d);
-            const int mine = (mt == mb) ? ct : 0;
+            const unsigned long long mb = block_min_u64(mt, red_u);
+            const int mine = (mt == mb && mb != ~0ull) ? ct : 0;
             int tot_b = 0;
-            const int ex = block_exclusive_scan(mine, red_i, &tot_b);
-            const int small_max = min(KS, T);
+            const int ex = block_scan_excl(mine, red_i, &tot_b);
+            const int small_max = min(KS, 1 << (31 - __clz(T)));  // a lane per particle at least
             if (mine > 0 && tot_b <= small_max) {
                 int pos = ex;
                 for (int i = c0; i < c1; ++i)
-                    if (a.t[i] + a.dt[i] == mb)
+                    if (static_cast<unsigned long long>(__double_as_longlong(a.t[i] + a.dt[i])) == mb)
                         s_cand[par][pos++] = i;
             }
             if (tid == 0) {
@@ -1039,63 +810,81 @@ __global__ void __launch_bounds__(kEnsThreads, 1) ensemble_kernel(EnsArgs a)
                 s_cnt2[par] = tot_b;
             }
             cl.sync();
-            double tn = INFINITY;
-            int fail = 0;
-            for (int r = 0; r < G; ++r) {
-                tn = fmin(tn, *cl.map_shared_rank(&s_min2[par], r));
-                fail |= *cl.map_shared_rank(&s_fail, r);
+            // every warp: lane r looks at block r
+            const int lane = tid & 31, rr = min(lane, G - 1);
+            const unsigned long long r_min = *cl.map_shared_rank(&s_min2[par], rr);
+            const int r_cnt = *cl.map_shared_rank(&s_cnt2[par], rr);
+            const bool fail = __any_sync(0xffffffffu, *cl.map_shared_rank(&s_fail, rr) != 0);
+            unsigned long long tn_bits = r_min;
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long u = __shfl_xor_sync(0xffffffffu, tn_bits, o);
+                tn_bits = u < tn_bits ? u : tn_bits;
             }
+            const double tn = __longlong_as_double(static_cast<long long>(tn_bits));
             if (tn > a.t_end || fail)
                 break;
-            int total = 0, prefix = 0;
-            for (int r = 0; r < G; ++r) {
-                const int v = (*cl.map_shared_rank(&s_min2[par], r) == tn) ? *cl.map_shared_rank(&s_cnt2[par], r) : 0;
-                prefix += r < rank ? v : 0;
-                total += v;
+            const int v_cnt = lane < G && r_min == tn_bits ? r_cnt : 0;
+            int incl = v_cnt;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o)
+                    incl += u;
             }
+            const int total = __shfl_sync(0xffffffffu, incl, 31);
+            const int prefix = __shfl_sync(0xffffffffu, incl - v_cnt, rank);
+            const int own_cnt = __shfl_sync(0xffffffffu, v_cnt, rank);
             if (total <= small_max) {
-                // active list in ascending order from the blocks' lists, and
-                // its predicted values (the arithmetic of the j-records)
-                if (tid < G) {
-                    const int v = (*cl.map_shared_rank(&s_min2[par], tid) == tn) ? *cl.map_shared_rank(&s_cnt2[par], tid) : 0;
-                    s_rcnt[tid] = v;
-                }
+                // active list in ascending order from the blocks' lists
+                if (tid < 32 && lane < G)
+                    s_rcnt[lane] = v_cnt;
                 __syncthreads();
                 for (int k = tid; k < total; k += T) {
                     int base = 0, r = 0;
                     while (k >= base + s_rcnt[r])
                         base += s_rcnt[r++];
-                    const int i = *cl.map_shared_rank(&s_cand[par][k - base], r);
-                    s_act[k] = i;
-                    store_ivalues<PR>(a, i, tn, s_iv[k]);
+                    s_act[k] = *cl.map_shared_rank(&s_cand[par][k - base], r);
                 }
                 __syncthreads();
                 if (a.log_cnt && rank == 0)
                     log_step(a, c, tn, total, s_act, off, &s_log_ip);
-                eval_small<PR>(a, lo, hi, tn, total, s_iv, s_part, s_wred, smem, 2 * a.jtile);
+                eval_small<PR>(a, lo, hi, tn, total, s_act, s_rec, KS, s_part, smem);
                 cl.sync();
-                for (int k = tid; k < total; k += T) {
-                    const int i = s_act[k];
-                    if (i < lo || i >= hi)
-                        continue;
-                    double f[9];
+                // this block's active particles: S threads per value add the
+                // blocks' partial sums, one adds theirs; then the corrector
+                double *sums = reinterpret_cast<double *>(smem);
+                CorrectScratch &scratch = *reinterpret_cast<CorrectScratch *>(smem + kSumBytes);
+                for (int o0 = 0; o0 < own_cnt; o0 += 32) {
+                    const int no = min(32, own_cnt - o0), nv = 9 * no;
+                    const int S = max(1, min(G, T / nv));
+                    for (int u = tid; u < nv * S; u += T) {
+                        const int v = u / S;
+                        double s4[4] = {0.0, 0.0, 0.0, 0.0};
+                        for (int r = u - v * S; r < G; r += 4 * S)
 #pragma unroll
-                    for (int q = 0; q < 9; ++q)
-                        f[q] = 0.0;
-                    for (int r = 0; r < G; ++r) {
-                        const double *pr = cl.map_shared_rank(&s_part[k][0], r);
-#pragma unroll
-                        for (int q = 0; q < 9; ++q)
-                            f[q] += pr[q];
+                            for (int e = 0; e < 4; ++e)
+                                if (r + e * S < G)
+                                    s4[e] += cl.map_shared_rank(s_part, r + e * S)[(prefix + o0) * 9 + v];
+                        sums[u] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
                     }
-                    correct_particle<PR>(a, i, tn, f);
+                    __syncthreads();
+                    if (S > 1) {
+                        const double s = tid < nv ? sum4(sums + tid * S, S) : 0.0;
+                        __syncthreads();
+                        if (tid < nv)
+                            sums[tid] = s;
+                        __syncthreads();
+                    }
+                    correct_few<PR>(a, s_act + prefix + o0, no, tn, sums, scratch);
+                    __syncthreads();
                 }
+                // the chunk area is also a TMA destination in later steps
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncthreads();
             } else {
-                if (mine > 0 && mb == tn) {
+                if (mine > 0 && mb == tn_bits) {
                     int pos = prefix + ex;
                     for (int i = c0; i < c1; ++i)
-                        if (a.t[i] + a.dt[i] == tn)
+                        if (static_cast<unsigned long long>(__double_as_longlong(a.t[i] + a.dt[i])) == mb)
                             a.act[off + pos++] = i;
                 }
                 predict_slice<PR>(a, lo, hi, tn);
@@ -1180,10 +969,14 @@ bool ens_mixed(const nb_ensemble *e)
     return e->cfg.precision == NB_MIXED || e->cfg.precision == NB_MIXED32;
 }
 
+// Two j-tiles; the same memory holds the lanes' sums (9 words of 8 bytes per
+// thread), then the summed forces of 32 particles and the corrector's scratch.
 size_t ens_smem(const nb_ensemble *e)
 {
     const int k = ens_kind(e);
-    return static_cast<size_t>(2) * (k == 1 || k == 3 ? NCF * 4 : (k == 2 ? NCX * 4 : 5 * 16)) * e->jtile;
+    const size_t tiles =
+        static_cast<size_t>(2) * (k == 1 || k == 3 ? NCF * 4 : (k == 2 ? NCX * 4 : 5 * 16)) * e->jtile;
+    return std::max({tiles, static_cast<size_t>(72) * e->threads, kSumBytes + sizeof(CorrectScratch)});
 }
 
 template <int PR>

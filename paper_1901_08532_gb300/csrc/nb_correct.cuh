@@ -6,6 +6,14 @@
 
 namespace nbk {
 
+// The criterion's value for quantise(): rounded down to a power of two from
+// FP32 logarithms where they decide, else in FP64.
+__device__ __forceinline__ double criterion(const double (&n2)[6], double eta)
+{
+    int k;
+    return aarseth_log2(n2, eta, &k) ? __hiloint2double((1023 + k) << 20, 0) : aarseth_dt(n2, eta);
+}
+
 // ------------------------------------------- corrector of one particle, FP64
 
 // Corrector, interpolation and new step of particle i at time t1 with its
@@ -27,7 +35,7 @@ __device__ __forceinline__ void correct_particle_fp64(double *st, double *t, dou
                                                       nb_ctl *ctl, double noise = 0.0)
 {
     const double h = t1 - t[i];
-    const double ih = 1.0 / h;  // exact: h is a power of two (the particle's step)
+    const double ih = inverse_step(h);  // exact: h is a power of two (the particle's step)
     double n2[6] = {0, 0, 0, 0, 0, 0};  // squared norms of a1, j1, s1, c1, d1, e1
     double m2[3] = {0, 0, 0};  // squared norms of a0, j0, s0 (their rounding floor)
     bool finite = true;
@@ -79,9 +87,7 @@ __device__ __forceinline__ void correct_particle_fp64(double *st, double *t, dou
         n2[4] = dd * dd;
         n2[5] = e * e;
     }
-    const double dtn =
-        dt_shared > 0.0 ? dt_shared : quantise(aarseth_dt(n2, eta), dt[i], t1, dt_min, dt_max, &hit);
-    dt[i] = dtn;
+    dt[i] = dt_shared > 0.0 ? dt_shared : quantise(criterion(n2, eta), dt[i], t1, dt_min, dt_max, &hit);
     if (hit)
         atomicAdd(reinterpret_cast<unsigned long long *>(&ctl->floor_hits), 1ull);
     if (!finite)
@@ -181,9 +187,7 @@ __device__ __forceinline__ void correct_group_fp64(double *st, double *t, double
         double dtn = dt_shared;
         if (!(dt_shared > 0.0)) {
             const double n2[6] = {sh.n2[0][l], sh.n2[1][l], sh.n2[2][l], sh.n2[3][l], sh.n2[4][l], sh.n2[5][l]};
-            int k;
-            const double crit = aarseth_log2(n2, eta, &k) ? __hiloint2double((1023 + k) << 20, 0) : aarseth_dt(n2, eta);
-            dtn = quantise(crit, dt[i], t1, dt_min, dt_max, &hit);
+            dtn = quantise(criterion(n2, eta), dt[i], t1, dt_min, dt_max, &hit);
         }
         dt[i] = dtn;
         if (hit)
