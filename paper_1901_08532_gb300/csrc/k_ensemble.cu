@@ -35,6 +35,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <functional>
 #include <numeric>
 #include <string>
 #include <vector>
@@ -1025,35 +1026,6 @@ cudaError_t max_clusters(nb_ensemble *e, int *out)
     return cudaOccupancyMaxActiveClusters(out, ensemble_kernel<PR>, &cfg);
 }
 
-// Default blocks per system: mixed ensembles 4 (their steps are latency-
-// bound); FP64 8; EX, whose steps carry most of the arithmetic at the FP32
-// rate, 16 where the device co-schedules clusters of 16 blocks, else 8.
-int default_ctas(nb_ensemble *e)
-{
-    if (ens_mixed(e))
-        return 4;
-    // FP64: 8 (with the j-split large-set path, smaller clusters run more
-    // systems at once and finish the largest ones no later: 256-system
-    // config 60.9 s against 66.7 s with 16)
-    if (e->cfg.precision == NB_FP64)
-        return 8;
-    const int keep = e->G;
-    e->G = 16;
-    int maxc = 0;
-    const cudaError_t err = ens_kind(e) == 2 ? max_clusters<2>(e, &maxc) : max_clusters<0>(e, &maxc);
-    e->G = keep;
-    if (err != cudaSuccess) {
-        (void)cudaGetLastError();
-        return 8;
-    }
-    return maxc >= 1 ? 16 : 8;
-}
-
-int default_jtile(const nb_ensemble *e) { return ens_mixed(e) ? 1024 : 256; }
-
-template <int PR>
-cudaError_t max_clusters(nb_ensemble *e, int *out);
-
 cudaError_t max_clusters_kind(nb_ensemble *e, int *out)
 {
     switch (ens_kind(e)) {
@@ -1063,6 +1035,86 @@ cudaError_t max_clusters_kind(nb_ensemble *e, int *out)
     default: return max_clusters<0>(e, out);
     }
 }
+
+// Default blocks per system, 4, 8 or 16: the choice with the smallest
+// estimated time of the queue (largest systems first).  A system of n particles
+// takes about 0.9 sqrt(n) steps and 2.2 n^2 interactions in the time that 256
+// to 2048 particles take for 1/64 (relative sizes matter, not this unit); a
+// step costs a fixed 20 us + 0.3 us per block, the interactions go at the
+// blocks' rate, which is a block's own where it has an SM to itself and a
+// share of the chip's where more blocks run than there are SMs, less what
+// splitting over G blocks loses.  Few systems want large clusters (the largest
+// system is the last to finish), many want small ones.  Measured with 4 / 8 /
+// 16 blocks (ms): FP64 32 systems of 256-2048 30.5 / 28.1 / 14.7 (8 before),
+// 100 of 256-1024 15.8 / 9.2 / 11.8, 256 of 256-16384 - / 60.9 / 66.6 s; mixed
+// 32 of 256-4096 6.9 / 4.8 / 3.8 (4 before), 128 10.1 / 6.2 / 10.5, 256 of
+// 256-16384 2.43 / 1.28 / 1.65 s; EX 100 of 256-1500 8.8 / 4.8 / 6.0 (16 before),
+// 256 of 256-16384 - / 11.3 / 11.1 s.  The estimate takes the best one in each.
+int default_ctas(nb_ensemble *e)
+{
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->dev) != cudaSuccess || sms < 1) {
+        (void)cudaGetLastError();
+        return 8;
+    }
+    // interactions per microsecond of a full SM and of a block alone on its
+    // SM, and the loss per block of a cluster
+    const bool ex = e->cfg.precision == NB_EX, mixed = ens_mixed(e);
+    const double full = mixed ? 2600.0 : ex ? 400.0 : 66.0, alone = mixed ? 1600.0 : ex ? 270.0 : 52.0;
+    const double loss = mixed ? 0.006 : ex ? 0.0 : 0.02;
+    std::vector<double> n(e->cnt.begin(), e->cnt.end());
+    std::sort(n.begin(), n.end(), std::greater<double>());
+    struct Running {
+        double left, fixed, work;  // fraction to go, latency part, interactions of a block
+    };
+    const int keep = e->G;
+    int best = 8;
+    double tbest = 1e300;
+    for (const int g : {4, 8, 16}) {
+        e->G = g;
+        int maxc = 0;
+        if (max_clusters_kind(e, &maxc) != cudaSuccess || maxc < 1) {
+            (void)cudaGetLastError();
+            continue;
+        }
+        std::vector<Running> run;
+        size_t next = 0;
+        auto start = [&]() {
+            const double k = n[next++];
+            run.push_back({1.0, 0.9 * std::sqrt(k) * (20.0 + 0.3 * g), 2.2 * k * k * (1.0 + loss * g) / g});
+        };
+        while (next < n.size() && run.size() < static_cast<size_t>(maxc))
+            start();
+        double t = 0.0;
+        while (!run.empty()) {
+            const double rate = std::min(alone, full * sms / (static_cast<double>(run.size()) * g));
+            size_t first = 0;
+            double dt = 1e300;
+            for (size_t q = 0; q < run.size(); ++q) {
+                const double need = run[q].left * (run[q].fixed + run[q].work / rate);
+                if (need < dt) {
+                    dt = need;
+                    first = q;
+                }
+            }
+            t += dt;
+            for (Running &r : run)
+                r.left -= dt / (r.fixed + r.work / rate);
+            run[first] = run.back();
+            run.pop_back();
+            if (next < n.size())
+                start();
+        }
+        if (t < 1.03 * tbest) {  // larger clusters where the estimates are alike
+            tbest = t;
+            best = g;
+        }
+    }
+    e->G = keep;
+    return best;
+}
+
+int default_jtile(const nb_ensemble *e) { return ens_mixed(e) ? 1024 : 256; }
 
 EnsArgs make_args(nb_ensemble *e, int mode, double t_end)
 {
@@ -1271,11 +1323,7 @@ nb_status nb_ensemble_init(nb_ensemble **out, int32_t n_systems, const int64_t *
     e->eps = eps;
     e->nc = n_systems;
     e->P = padded;
-    // defaults from shape sweeps on GB300: mixed 4 x 128 threads, j-tile
-    // 1024; FP64 and EX 16 (or 8) x 128, j-tile 256 (set below, once the
-    // device is known)
     e->jtile = default_jtile(e);
-    e->G = ens_mixed(e) ? 4 : 8;
     auto bail = [&](nb_status s) {
         nb_set_thread_error(e->err.c_str());
         ens_free_all(e);
@@ -1297,7 +1345,6 @@ nb_status nb_ensemble_init(nb_ensemble **out, int32_t n_systems, const int64_t *
         EI(cudaStreamCreateWithFlags(&e->stream, cudaStreamNonBlocking));
         e->own_stream = true;
     }
-    e->G = default_ctas(e);
     e->off.resize(n_systems);
     e->cnt.resize(n_systems);
     {
@@ -1310,6 +1357,7 @@ nb_status nb_ensemble_init(nb_ensemble **out, int32_t n_systems, const int64_t *
     }
     for (int c = 0; c < n_systems; ++c)
         e->nmax4 = std::max<int64_t>(e->nmax4, (e->cnt[c] + 3) / 4 * 4);
+    e->G = default_ctas(e);
     std::vector<int32_t> order(n_systems);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(),

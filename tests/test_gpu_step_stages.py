@@ -114,3 +114,27 @@ def test_device_steps_match_host_steps_at_launch_edges(prec, n):
     for k, tol in (("x", 1e-12), ("v", 1e-12), ("a", 1e-11), ("j", 1e-10)):
         tol = tol if prec != 1 else (1e-9 if k in "xv" else 1e-5)
         assert np.abs(a[k] - b[k]).max() <= tol * np.abs(b[k]).max(), k
+
+
+@pytest.mark.parametrize("prec", [0, 3])
+@pytest.mark.parametrize("shape", [(4, 64, 16), (8, 96, 64), (4, 160, 128), (16, 256, 256), (3, 128, 8)])
+def test_ensemble_shapes_take_the_same_steps(prec, shape):
+    """Block and lane counts that are no power of two, j-tiles smaller than the scratch that shares their memory:
+    the decisions of the default shape, and its state to the rounding of another summation order."""
+    nb = nb_gpu()
+    sizes = np.array([5, 130, 301, 64])
+    m, x, v = (np.concatenate([ni.plummer(int(k), 40 + q)[f] for q, k in enumerate(sizes)]) for f in range(3))
+    out = []
+    for sh in (None, shape):
+        e = nb.Ensemble(sizes, m, x, v, 1e-2, precision=prec, dt_max=2.0 ** -6)
+        if sh:
+            e.set_shape(*sh)
+        e.run(2.0 ** -6)
+        out.append((e.stats()[0], e.state()))
+        e.close()
+    (sa, a), (sb, b) = out
+    np.testing.assert_array_equal(sa, sb)
+    np.testing.assert_array_equal(a["t"], b["t"])
+    np.testing.assert_array_equal(a["dt"], b["dt"])
+    for k, tol in (("x", 1e-12), ("v", 1e-12), ("a", 1e-11), ("j", 1e-10)):
+        assert np.abs(a[k] - b[k]).max() <= tol * np.abs(b[k]).max(), k
