@@ -119,10 +119,9 @@ typedef struct {
     int32_t device_steps; /* 1: nb_run_until and nb_run_diag run block steps
                           whose active set holds at most 128 particles inside
                           one cooperative launch (device-resident scheduling,
-                          evaluation and correction; larger steps return to
-                          the host-driven path, and after a launch that took
-                          no step the host tries again only after 1, 3, 7 ...
-                          host steps); 0: every step host-driven            */
+                          evaluation and correction; a larger step returns to
+                          the host-driven path with its active set listed);
+                          0: every step host-driven                         */
     double step_noise;  /* 0: the generalised Aarseth criterion as is.  > 0:
                           the relative rounding level of the evaluated a,
                           jerk and snap (about 4e-7 = 2^-21 for NB_MIXED,

@@ -101,6 +101,23 @@ __global__ void transpose_kernel(const double *anew, int ostride, int n_act, int
     dst[e] = anew[(q0 + d) * (size_t)ostride + k];
 }
 
+// All nine rows of anew -> acc, jerk, snap [n_act][3] (NULL: not wanted), in one
+// launch: small evaluations are bound by the number of launches.
+__global__ void __launch_bounds__(256) outputs_kernel(const double *anew, int ostride, int n_act, double *acc,
+                                                      double *jerk, double *snap)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n_act)
+        return;
+    double *const dst[3] = {acc, jerk, snap};
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+        if (dst[q])
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                dst[q][3 * static_cast<size_t>(k) + d] = anew[(3 * q + d) * static_cast<size_t>(ostride) + k];
+}
+
 // State layout conversions: [n][3] rows (the C-ABI's vector layout) <->
 // three component rows of the structure-of-arrays state.
 __global__ void rows_to_soa_kernel(const double *rows, double *soa, int n)
@@ -172,6 +189,15 @@ cudaError_t nb_launch_init_state(nb_ctx *c, int pass)
     init_state_kernel<<<(n + 127) / 128, 128, 0, c->stream>>>(c->st, c->dt, c->anew, n, pass,
                                                                c->cfg.eta_s, c->cfg.dt_min,
                                                                c->cfg.dt_max, c->cfg.dt_shared, c->ctl);
+    c->launches += 1;
+    return cudaGetLastError();
+}
+
+cudaError_t nb_launch_outputs(nb_ctx *c, int n_act, double *acc, double *jerk, double *snap)
+{
+    if (n_act <= 0 || (!acc && !jerk && !snap))
+        return cudaSuccess;
+    outputs_kernel<<<(n_act + 255) / 256, 256, 0, c->stream>>>(c->anew, static_cast<int>(c->n), n_act, acc, jerk, snap);
     c->launches += 1;
     return cudaGetLastError();
 }

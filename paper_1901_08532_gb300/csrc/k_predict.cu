@@ -87,7 +87,6 @@ cudaError_t nb_launch_predict(nb_ctx *c, double t)
     const int n = static_cast<int>(c->n);
     const int block = 256;
     int grid = (n + block - 1) / block;
-    grid = grid < c->sm_count * 16 ? grid : c->sm_count * 16;
     const bool rows = nb_jrows(c->cfg.precision) > 0;
     const int mode = c->cfg.precision == NB_EX ? kModeEx : (c->cfg.precision == NB_SP ? kModeSp : kModeMixed);
     predict_kernel<<<grid, block, 0, c->stream>>>(c->st, c->t, c->m, n, t, rows ? nullptr : c->jb64,

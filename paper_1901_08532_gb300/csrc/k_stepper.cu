@@ -27,8 +27,8 @@
 // per step with about 13 active particles, before -> after: FP64 N = 1024
 // 39.2 -> 18.1 us, EX N = 8192 46.1 -> 20.7 us, mixed N = 65536 58.0 -> 31.6 us.
 // It returns to the host when the next active set holds more than
-// kStepSmall particles (the host then runs that step with the tuned
-// evaluation kernels), when the next block time passes t_end, or after an
+// kStepSmall particles, which it leaves listed (the host then runs that step
+// with the tuned evaluation kernels and needs no scheduler pass, about 28 us), when the next block time passes t_end, or after an
 // error flag.  Every block takes the same branch at every barrier (decisions
 // come from the same global values), and no block waits on a flag.
 #include <cooperative_groups.h>
@@ -63,6 +63,8 @@ struct StepOut {
     int32_t reason;    // 0: next block time beyond t_end, 1: next active set too large, 2: error
     int32_t n_act;     // active count of the last step taken
     double t_last;     // time of the last step taken
+    double t_next;     // reason 1: time of the next step and its active count
+    int32_t n_next;
 };
 
 struct StepArgs {
@@ -76,6 +78,7 @@ struct StepArgs {
     int *cand;          // [B][kStepSmall] their indices, ascending
     double *part;       // [kStepSmall][9][B] partial sums
     int32_t *act;       // active set of the last step taken
+    int32_t *act_next;  // reason 1: the next active set, ascending
     nb_ctl *ctl;
     StepOut *out;
     double *log_t;      // per-step log (device), entries [log_base, log_cap)
@@ -100,8 +103,8 @@ __global__ void __launch_bounds__(T) step_kernel(StepArgs a)
     const int per_t = (hi - lo + T - 1) / T;
     const int c0 = min(hi, lo + tid * per_t), c1 = min(hi, c0 + per_t);
     int64_t steps = 0, act_sum = 0;
-    int reason = 0, last_n = 0;
-    double last_t = 0.0;
+    int reason = 0, last_n = 0, next_n = 0;
+    double last_t = 0.0, next_t = 0.0;
     for (;;) {
         // schedule: this block's earliest t_i + dt_i, the particles reaching it
         unsigned long long mt = ~0ull;
@@ -147,7 +150,7 @@ __global__ void __launch_bounds__(T) step_kernel(StepArgs a)
         int c = 0;
 #pragma unroll
         for (int e = 0; e < kQ; ++e)
-            c += bm[e] == mn_bits ? min(bc[e], kStepSmall + 1) : 0;
+            c += bm[e] == mn_bits ? bc[e] : 0;
         int total = 0;
         int pos = block_scan_excl(c, red_i, &total);
         if (err) {
@@ -159,7 +162,24 @@ __global__ void __launch_bounds__(T) step_kernel(StepArgs a)
             break;
         }
         if (total > kStepSmall) {
+            // too many for a step here: list them for the host's
             reason = 1;
+            __syncthreads();  // red_i was read by the scan
+#pragma unroll
+            for (int e = 0, q = pos; e < kQ; ++e) {
+                if (tid * kQ + e == bk)
+                    red_i[0] = q;
+                q += bm[e] == mn_bits ? bc[e] : 0;
+            }
+            __syncthreads();
+            if (mine > 0 && mb == mn_bits) {
+                int at = red_i[0] + ex;
+                for (int i = c0; i < c1; ++i)
+                    if (static_cast<unsigned long long>(__double_as_longlong(a.t[i] + a.dt[i])) == mb)
+                        a.act_next[at++] = i;
+            }
+            next_t = mn;
+            next_n = total;
             break;
         }
         // active list, ascending: blocks in order, each block's list in order
@@ -248,6 +268,8 @@ __global__ void __launch_bounds__(T) step_kernel(StepArgs a)
         a.out->reason = reason;
         a.out->n_act = last_n;
         a.out->t_last = last_t;
+        a.out->t_next = next_t;
+        a.out->n_next = next_n;
     }
 }
 
@@ -280,10 +302,10 @@ cudaError_t launch_stepper(nb_ctx *c, StepArgs &a, int grid_max)
 
 int nb_stepper_small() { return kStepSmall; }
 
-// One launch of the device-resident stepper; reports what it did in
-// *steps, *act_sum, *reason, *n_act, *t_last (synchronises the stream).
-cudaError_t nb_run_stepper(nb_ctx *c, double t_end, int64_t log_cap, int64_t log_base, int64_t *steps,
-                           int64_t *act_sum, int *reason, int *n_act, double *t_last)
+// One launch of the device-resident stepper; reports what it did in *r
+// (synchronises the stream).  reason 1 leaves the next active set in
+// c->act_next.
+cudaError_t nb_run_stepper(nb_ctx *c, double t_end, int64_t log_cap, int64_t log_base, StepperResult *r)
 {
     // scratch sized for the largest grid this device can hold
     const int grid_max = c->sm_count * 16;
@@ -318,6 +340,7 @@ cudaError_t nb_run_stepper(nb_ctx *c, double t_end, int64_t log_cap, int64_t log
     a.cand = c->stp_cand;
     a.part = c->stp_part;
     a.act = c->act;
+    a.act_next = c->act_next;
     a.ctl = c->ctl;
     a.out = static_cast<StepOut *>(c->stp_out);
     a.log_t = c->stp_log_t;
@@ -337,10 +360,6 @@ cudaError_t nb_run_stepper(nb_ctx *c, double t_end, int64_t log_cap, int64_t log
     if (e != cudaSuccess)
         return e;
     const StepOut *o = static_cast<const StepOut *>(c->stp_out_h);
-    *steps = o->steps;
-    *act_sum = o->act_sum;
-    *reason = o->reason;
-    *n_act = o->n_act;
-    *t_last = o->t_last;
+    *r = {o->steps, o->act_sum, o->reason, o->n_act, o->t_last, o->t_next, o->n_next};
     return cudaSuccess;
 }

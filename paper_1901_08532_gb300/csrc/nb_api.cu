@@ -233,22 +233,19 @@ nb_status integrate_to(nb_ctx *c, double t_end, int64_t log_cap, double *log_t, 
         c->stp_log_n = nullptr;
     };
     nb_status s = NB_OK;
-    int backoff = 0, skip = 0;  // host steps before the stepper is tried again
     for (;;) {
-        if (device && skip > 0) {
-            --skip;
-        } else if (device) {
-            int64_t ds = 0, acts = 0;
-            int reason = 0, na_last = 0;
-            double t_last = 0.0;
-            cudaError_t e = nb_run_stepper(c, t_end, log_cap, steps, &ds, &acts, &reason, &na_last, &t_last);
+        double tn = 0.0;  // the next step, once known
+        int64_t na = 0;
+        if (device) {
+            StepperResult r{};
+            cudaError_t e = nb_run_stepper(c, t_end, log_cap, steps, &r);
             if (e != cudaSuccess) {
                 release_log();
                 return cuda_fail(c, e, "device-resident block steps");
             }
-            if (ds > 0) {
+            if (r.steps > 0) {
                 if (log_cap > steps) {
-                    const int64_t k = std::min(ds, log_cap - steps);
+                    const int64_t k = std::min(r.steps, log_cap - steps);
                     e = cudaMemcpyAsync(log_t + steps, c->stp_log_t + steps, k * sizeof(double),
                                         cudaMemcpyDeviceToHost, c->stream);
                     if (e == cudaSuccess)
@@ -261,25 +258,23 @@ nb_status integrate_to(nb_ctx *c, double t_end, int64_t log_cap, double *log_t, 
                         return cuda_fail(c, e, "step log copy");
                     }
                 }
-                steps += ds;
-                c->t_sys = t_last;
-                c->n_act = na_last;
-                c->interactions += static_cast<double>(acts) * static_cast<double>(c->n);
+                steps += r.steps;
+                c->t_sys = r.t_last;
+                c->n_act = r.n_act;
+                c->interactions += static_cast<double>(r.act_sum) * static_cast<double>(c->n);
             }
-            if (reason != 1)
+            if (r.reason != 1)
                 break;  // t_end reached, or an error flag (reported by sync_ctl)
-            // the next active set is too large: a launch that took no step at
-            // all doubles the number of host steps before the next attempt
-            backoff = ds > 0 ? 0 : std::min(2 * backoff + 1, 255);
-            skip = backoff;
+            // the next active set is too large for it, and listed in c->act_next
+            tn = r.t_next;
+            na = r.n_next;
+        } else {
+            s = schedule(c, &tn, &na);
+            if (s != NB_OK)
+                break;
+            if (tn > t_end)
+                break;
         }
-        double tn;
-        int64_t na;
-        s = schedule(c, &tn, &na);
-        if (s != NB_OK)
-            break;
-        if (tn > t_end)
-            break;
         if (na < 1) {
             s = fail(c, NB_ESTATE, "scheduler found no active particle");
             break;
@@ -595,18 +590,16 @@ nb_status nb_evaluate(nb_ctx *c, const int32_t *active, int64_t n_act, int activ
     c->t_eval = c->t_pred;
     double *outs[3] = {acc, jerk, snap};
     bool host_copy = false;
-    for (int q = 0; q < 3; ++q) {
+    if (out_on_device)
+        CU(c, nb_launch_outputs(c, static_cast<int>(n_act), acc, jerk, snap));
+    for (int q = 0; q < 3 && !out_on_device; ++q) {
         if (!outs[q] || n_act == 0)
             continue;
-        if (out_on_device) {
-            CU(c, nb_launch_transpose_out(c, static_cast<int>(n_act), 3 * q, outs[q]));
-        } else {
-            CU(c, nb_launch_transpose_out(c, static_cast<int>(n_act), 3 * q, c->stage));
-            CU(c, cudaMemcpyAsync(outs[q], c->stage, static_cast<size_t>(3 * n_act) * sizeof(double),
-                                  cudaMemcpyDeviceToHost, c->stream));
-            CU(c, cudaStreamSynchronize(c->stream));
-            host_copy = true;
-        }
+        CU(c, nb_launch_transpose_out(c, static_cast<int>(n_act), 3 * q, c->stage));
+        CU(c, cudaMemcpyAsync(outs[q], c->stage, static_cast<size_t>(3 * n_act) * sizeof(double),
+                              cudaMemcpyDeviceToHost, c->stream));
+        CU(c, cudaStreamSynchronize(c->stream));
+        host_copy = true;
     }
     if (host_copy)
         return sync_ctl(c);

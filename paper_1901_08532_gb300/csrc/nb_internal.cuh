@@ -253,7 +253,9 @@ cudaError_t nb_launch_predict(nb_ctx *c, double t);
 // k_correct.cu
 cudaError_t nb_launch_correct(nb_ctx *c, double t1, int n_act);
 cudaError_t nb_launch_init_state(nb_ctx *c, int pass);
+// anew rows q0 .. q0 + 2 -> dst [n_act][3]; all three sums where wanted (NULL: not)
 cudaError_t nb_launch_transpose_out(nb_ctx *c, int n_act, int q0, double *dst);
+cudaError_t nb_launch_outputs(nb_ctx *c, int n_act, double *acc, double *jerk, double *snap);
 cudaError_t nb_launch_rows_to_soa(nb_ctx *c, const double *rows, int field);
 cudaError_t nb_launch_soa_to_rows(nb_ctx *c, int field, double *rows);
 // k_sched.cu
@@ -263,8 +265,15 @@ cudaError_t nb_launch_iota(nb_ctx *c, int n, int32_t *dst);
 void nb_set_thread_error(const char *msg);
 // k_stepper.cu
 int nb_stepper_small();
-cudaError_t nb_run_stepper(nb_ctx *c, double t_end, int64_t log_cap, int64_t log_base, int64_t *steps,
-                           int64_t *act_sum, int *reason, int *n_act, double *t_last);
+struct StepperResult {
+    int64_t steps, act_sum;  // block steps taken and the active particles summed over them
+    int reason;              // 0: t_end reached, 1: next active set too large, 2: error flag
+    int n_act;               // active count and time of the last step taken
+    double t_last;
+    double t_next;           // reason 1: time and active count of the next step
+    int n_next;
+};
+cudaError_t nb_run_stepper(nb_ctx *c, double t_end, int64_t log_cap, int64_t log_base, StepperResult *r);
 
 // k_energy.cu
 cudaError_t nb_launch_energy(nb_ctx *c, double *ek_pe_dev);
