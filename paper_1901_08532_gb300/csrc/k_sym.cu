@@ -4,7 +4,7 @@
 // and beta.  Swapping i and j negates r, v and a, keeps alpha and beta, and
 // so negates u and w: the terms on j are (-m_i / m_j) times those on i.  Per
 // unordered pair the mixed formula takes 63 FP32-pipe operations instead of
-// 2 x 53 (FP64 63 instead of 106, EX 608 instead of 992).
+// 2 x 53 (FP64 60 instead of 100, EX 608 instead of 992).
 //
 // Work split.  The particles form T tiles of B; a job (b, d) is the pairs of
 // tile b with tile (b + d) mod T, and d = 0 .. T/2 covers every unordered pair
@@ -426,7 +426,7 @@ __device__ __forceinline__ void pair_fp64_sym(const double2 (&c)[5], const doubl
     const double mu = c[1].y * q3, nu = nmi * q3;
     const double al = rv * q2;
     const double be = fma(al, al, sv * q2);
-    const double a3 = 3.0 * al, a6 = 6.0 * al, b3 = 3.0 * be;
+    const double a3 = 3.0 * al, a6 = twice(a3), b3 = 3.0 * be;
     const double ux = fma(-a3, dx, dvx), uy = fma(-a3, dy, dvy), uz = fma(-a3, dz, dvz);
     const double wx = fma(-a6, ux, fma(-b3, dx, dax));
     const double wy = fma(-a6, uy, fma(-b3, dy, day));
@@ -439,12 +439,12 @@ __device__ __forceinline__ void pair_fp64_sym(const double2 (&c)[5], const doubl
     }
 }
 
-// Bound by the FP64 pipe (94 % of 2 operations per clock and SM): 63 operations
-// per unordered pair for 106, so loads and shuffles cost nothing.  One warp per
+// Bound by the FP64 pipe (93 % of 2 operations per clock and SM): 60 operations
+// per unordered pair for 100, so loads and shuffles cost nothing.  One warp per
 // scheduler fills the pipe; W = 1 and 2 give small systems enough blocks.
-// All particles, ordinary kernel -> this one: 1000 114 -> 96 us, 2000 402 ->
-// 275, 4096 1.58 -> 0.98 ms, 8191 6.24 -> 3.87, 30000 84.9 -> 50.3 ms
-// (1.79e10 interactions/s).  Below about 900 particles the ordinary kernel is
+// All particles, ordinary kernel -> this one: 1000 112 -> 94 us, 2000
+// 394 -> 266, 4096 1.54 -> 0.95 ms, 8191 6.10 -> 3.73, 30000 82.9 -> 48.4 ms (1.86e10
+// interactions/s).  Below about 900 particles the ordinary kernel is
 // faster.
 template <int W>
 __global__ void __launch_bounds__(32 * W) sym_fp64_kernel(SymArgs a)

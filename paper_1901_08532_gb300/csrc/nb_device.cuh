@@ -38,7 +38,7 @@ __device__ __forceinline__ void pair_fp64(const double2 &p0, const double2 &p1, 
     const double mu = mj * q * q2;
     const double al = rv * q2;
     const double be = fma(al, al, sv * q2);
-    const double a3 = 3.0 * al, a6 = 6.0 * al, b3 = 3.0 * be;
+    const double a3 = 3.0 * al, a6 = nbk::twice(a3), b3 = 3.0 * be;
     const double ux = fma(-a3, dx, dvx), uy = fma(-a3, dy, dvy), uz = fma(-a3, dz, dvz);
     const double wx = fma(-a6, ux, fma(-b3, dx, dax));
     const double wy = fma(-a6, uy, fma(-b3, dy, day));

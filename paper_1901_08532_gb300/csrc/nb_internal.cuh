@@ -187,27 +187,56 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
 
 constexpr unsigned long long kWaitLimitNs = 1000000000ull;  // 1 s
 
-// Reciprocal square root of a positive normal double: an FP32 hardware
-// estimate (inputs and result converted by exponent re-biasing on the
-// integer pipe) refined by one third-order Householder step,
-//   y = y0 (1 + h/2 + 3 h^2 / 8),  h = 1 - x y0^2,
-// the series of (1 - h)^(-1/2) truncated after h^2.  From a 2^-22 estimate
-// the truncation error is below 2^-63, so the result is within about one
-// rounding of 1/sqrt(x).  Valid for 2^-126 < x < 2^127 (FP32 normal range).
+// Reciprocal square root of a positive normal double in three FP64 operations
+// (the FP64 pipe runs at 1/64 of FP32 here; an FP32 seed alone takes five for a
+// third-order step).  x = m 4^k with m in [1, 4); y = the FP32 hardware estimate
+// of 1/sqrt(m); its residual r = 1 - m y^2 in FP32 (y^2 exactly as a pair, m as
+// a pair) gives the correction y r / 2, added to y's bits as an integer and
+// rounded to 26 bits: y0, within 2^-26.  Then y0^2 is exact, h = 1 - x y0^2
+// rounds once, and y = y0 + (y0 / 2)(1 + 3 h / 4) h, the series of
+// (1 - h)^(-1/2) to h^2 (what is left is below 2^-75), rounds once more: the
+// factor 1 + 3 h / 4 goes into the bits of y0 / 2 as an integer too.
+// Valid for all positive normal x; relative error within 1.0 x 2^-53, rms 0.43.
+// Against the five-operation form: 8191 particles in FP64 3.87 -> 3.73 ms, the
+// energy of 131072 186 -> 153 ms.
 __device__ __forceinline__ double rsqrt_fp64(double x)
 {
-    const int hi = __double2hiint(x);
-    const unsigned lo = static_cast<unsigned>(__double2loint(x));
-    // double (11-bit exponent, bias 1023) -> float (8-bit, bias 127), mantissa truncated
-    const unsigned fb = (static_cast<unsigned>(hi - (896 << 20)) << 3) | (lo >> 29);
-    float yf;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(__uint_as_float(fb)));
-    const unsigned yb = __float_as_uint(yf);
-    const double y0 = __hiloint2double(static_cast<int>((yb >> 3) + (896u << 20)),
-                                       static_cast<int>(yb << 29));
+    const unsigned hi = static_cast<unsigned>(__double2hiint(x)), lo = static_cast<unsigned>(__double2loint(x));
+    const unsigned odd = ~(hi >> 20) & 1u;  // of the unbiased exponent (bias 1023)
+    // m = mh + ml, mh the leading 24 bits
+    const float mh = __uint_as_float(((hi & 0xfffffu) << 3 | lo >> 29) + ((127u + odd) << 23));
+    const float ml = static_cast<float>(lo & 0x1fffffffu) * (odd ? 0x1p-51f : 0x1p-52f);
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(mh));
+    y = fmaxf(fminf(y, 0x1.fffffep-1f), 0.5f);  // one binade, [1/2, 1): units of 2^-24
+    const float p = __fmul_rn(y, y), e = __fmaf_rn(y, y, -p);
+    const float r = __fmaf_rn(-ml, p, __fmaf_rn(-mh, e, __fmaf_rn(-mh, p, 1.0f)));
+    // y + y r / 2 in units of 2^-26: four per unit of y
+    const int c = __float2int_rn(__fmul_rn(__fmul_rn(y, r), 0x1p25f));
+    const unsigned yb = __float_as_uint(y);
+    long long bits = (static_cast<long long>((yb >> 3) + (896u << 20)) << 32 | static_cast<long long>(yb << 29)) +
+                     static_cast<long long>(c) * (1ll << 27);
+    // exponent: y0 = y 2^-k, k = (E - odd) / 2 with E the unbiased exponent
+    bits -= static_cast<long long>((static_cast<int>(hi >> 20) - 1023 - static_cast<int>(odd)) / 2) * (1ll << 52);
+    const double y0 = __longlong_as_double(bits);
     const double h = fma(-x, y0 * y0, 1.0);
-    const double p = fma(h, 0.375, 0.5);
-    return fma(h * y0, p, y0);
+    // |h| 2^53 as a float from h's bits (0 where h is too small to matter)
+    const int hh = __double2hiint(h);
+    const unsigned sh = 1023u - ((static_cast<unsigned>(hh) >> 20) & 0x7ff);  // |h| = 1.f 2^-sh
+    const float hm = __uint_as_float((static_cast<unsigned>(hh) & 0xfffffu) << 3 | 127u << 23);  // 1.f
+    const float hs = sh < 64u ? __fmul_rn(hm, __uint_as_float((127u + 53u - sh) << 23)) : 0.0f;   // |h| 2^53
+    const int d = __float2int_rn(__fmul_rn(__fmul_rn(y, 0.75f), hs));
+    const double half = __longlong_as_double(bits - (1ll << 52) + (hh < 0 ? -d : d));
+    return fma(half, h, y0);
+}
+
+// 2 x by the exponent, off the FP64 pipe.
+__device__ __forceinline__ double twice(double x)
+{
+    const int hi = __double2hiint(x);
+    if (static_cast<unsigned>((hi & 0x7ff00000) - 0x00100000) >= 0x7fd00000u)
+        return x + x;  // zero, subnormal, the largest, infinite, NaN
+    return __hiloint2double(hi + 0x00100000, __double2loint(x));
 }
 
 // TwoSum (Knuth): s + e == a + b exactly.  Accumulates the rounding error
