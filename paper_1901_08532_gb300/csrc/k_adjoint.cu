@@ -43,14 +43,20 @@ using namespace nbk;
 constexpr int kAdjThreads = 128;
 constexpr int kAdjTile = 64;
 
+// -3 alpha, -6 alpha and -3 beta of a pair.
+struct PairFactors {
+    double na3, na6, nb3;
+};
+
 // The bracket B(g) of dL/d(r, v, a) = q^3 B(g) for a pair with unit source
 // mass (mu = m_j q^3 factored out), linear in the cotangents g; phi = Phi(g).
+// Doublings go by the exponent, off the FP64 pipe (twice).
 __device__ __forceinline__ void bracket_from_phi(const double (&r)[3], const double (&v)[3], const double (&a)[3],
-                                                 double q2, double al, double be, double phi, const double *g,
-                                                 double (&br)[3], double (&bv)[3], double (&ba)[3])
+                                                 double q2, double al, double be, const PairFactors &k, double phi,
+                                                 const double *g, double (&br)[3], double (&bv)[3], double (&ba)[3])
 {
     const double *Ab = g, *Jb = g + 3, *Sb = g + 6;
-    const double c18 = 18.0 * al * al - 3.0 * be;
+    const double c18 = fma(k.na3, k.na6, k.nb3);  // 18 alpha^2 - 3 beta
     double sr = 0, sv = 0, jr = 0;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -58,29 +64,18 @@ __device__ __forceinline__ void bracket_from_phi(const double (&r)[3], const dou
         sv = fma(Sb[d], v[d], sv);
         jr = fma(Jb[d], r[d], jr);
     }
-    const double Pa = -3.0 * jr - 6.0 * sv + 36.0 * al * sr;
-    const double Pb = -3.0 * sr;
-    const double cv = fma(2.0 * al, Pb, Pa);
-    const double cr = fma(3.0, phi, fma(2.0 * al, Pa, 2.0 * (be + al * al) * Pb));
+    const double Pa = -3.0 * (jr + twice(fma(k.na6, sr, sv)));
+    const double Pb = -3.0 * sr, Pb2 = twice(Pb);
+    const double cv = fma(k.na6, sr, Pa);
+    const double ncr = -fma(3.0, phi, twice(fma(al, Pa, fma(al, al, be) * Pb)));
+    const double qPb = q2 * Pb;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        const double Pr = fma(c18, Sb[d], fma(-3.0 * al, Jb[d], Ab[d]));
-        br[d] = fma(q2, fma(cv, v[d], fma(Pb, a[d], -cr * r[d])), Pr);
-        bv[d] = fma(q2, fma(cv, r[d], 2.0 * Pb * v[d]), fma(-6.0 * al, Sb[d], Jb[d]));
-        ba[d] = fma(q2 * Pb, r[d], Sb[d]);
+        const double Pr = fma(c18, Sb[d], fma(k.na3, Jb[d], Ab[d]));
+        br[d] = fma(q2, fma(cv, v[d], fma(Pb, a[d], ncr * r[d])), Pr);
+        bv[d] = fma(q2, fma(cv, r[d], Pb2 * v[d]), fma(k.na6, Sb[d], Jb[d]));
+        ba[d] = fma(qPb, r[d], Sb[d]);
     }
-}
-
-__device__ __forceinline__ void pair_bracket(const double (&r)[3], const double (&v)[3], const double (&a)[3],
-                                             const double (&u)[3], const double (&w)[3], double q2, double al,
-                                             double be, const double *g, double (&br)[3], double (&bv)[3],
-                                             double (&ba)[3])
-{
-    double phi = 0;
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-        phi = fma(g[d], r[d], fma(g[3 + d], u[d], fma(g[6 + d], w[d], phi)));
-    bracket_from_phi(r, v, a, q2, al, be, phi, g, br, bv, ba);
 }
 
 // For particle k and every l: the pair (i = k, j = l) with k's cotangents and
@@ -149,10 +144,12 @@ __global__ void __launch_bounds__(kAdjThreads) adjoint_kernel(int n, int lanes, 
             const double be = fma(fma(vr[0], vr[0], fma(vr[1], vr[1], vr[2] * vr[2])) +
                                       fma(r[0], ar[0], fma(r[1], ar[1], r[2] * ar[2])),
                                   q2, al * al);
+            const double na3 = -3.0 * al;
+            const PairFactors f = {na3, twice(na3), -3.0 * be};
             double u[3], w[3];
             for (int d = 0; d < 3; ++d) {
-                u[d] = fma(-3.0 * al, r[d], vr[d]);
-                w[d] = fma(-6.0 * al, u[d], fma(-3.0 * be, r[d], ar[d]));
+                u[d] = fma(f.na3, r[d], vr[d]);
+                w[d] = fma(f.na6, u[d], fma(f.nb3, r[d], ar[d]));
             }
             const double ml = s_st[e][9];
             double gs[9];
@@ -161,8 +158,10 @@ __global__ void __launch_bounds__(kAdjThreads) adjoint_kernel(int n, int lanes, 
                 gs[q9] = fma(mk, s_g[e][q9], -ml * gk[q9]);
             for (int d = 0; d < 3; ++d)
                 phil = fma(s_g[e][d], r[d], fma(s_g[e][3 + d], u[d], fma(s_g[e][6 + d], w[d], phil)));
-            double br[3], bv[3], ba[3];
-            pair_bracket(r, vr, ar, u, w, q2, al, be, gs, br, bv, ba);
+            double br[3], bv[3], ba[3], phi = 0.0;
+            for (int d = 0; d < 3; ++d)
+                phi = fma(gs[d], r[d], fma(gs[3 + d], u[d], fma(gs[6 + d], w[d], phi)));
+            bracket_from_phi(r, vr, ar, q2, al, be, f, phi, gs, br, bv, ba);
             for (int d = 0; d < 3; ++d) {
                 ox[d] = fma(q3, br[d], ox[d]);
                 ov[d] = fma(q3, bv[d], ov[d]);
@@ -194,10 +193,11 @@ __global__ void __launch_bounds__(kAdjThreads) adjoint_kernel(int n, int lanes, 
 // to x_k, v_k, a_k and, negated, that with respect to x_l, v_l, a_l (swapping the
 // two negates g* and r, v, a, and the bracket with them), and Phi(g*) =
 // m_k Phi(g_l) - m_l Phi(g_k) comes from the two forms that the mass gradients
-// need.  About 165 FP64 operations per unordered pair instead of 2 x 150.
-// Bound by the FP64 pipe; the tile shrinks with W for small systems.
-// Ordered kernel -> this one: 700 particles 226 -> 185 us, 1000 326 -> 197,
-// 4096 4.47 -> 2.44 ms, 16384 71.0 -> 37.8 ms.
+// need.  About 150 FP64 operations per unordered pair instead of 2 x 140.
+// Bound by the FP64 pipe (87 % of 2 operations per clock and SM); the tile
+// shrinks with W for small systems.
+// Ordered kernel -> this one: 1000 particles 326 -> 195 us,
+// 4096 4.47 -> 2.37 ms, 8192 17.8 -> 9.35 ms.
 template <int W>
 __global__ void __launch_bounds__(32 * W) adjoint_sym_kernel(SymArgs a, const double *__restrict__ m,
                                                              const double *__restrict__ x,
@@ -274,12 +274,14 @@ __global__ void __launch_bounds__(32 * W) adjoint_sym_kernel(SymArgs a, const do
                                           fma(r[0], ar[0], fma(r[1], ar[1], r[2] * ar[2])),
                                       q2, al * al);
                 const double ml = tile[9][e];
+                const double na3 = -3.0 * al;
+                const PairFactors f = {na3, twice(na3), -3.0 * be};
                 double u[3], ww[3], gs[9];
                 double phil = 0.0, phik = 0.0;
 #pragma unroll
                 for (int d = 0; d < 3; ++d) {
-                    u[d] = fma(-3.0 * al, r[d], vr[d]);
-                    ww[d] = fma(-6.0 * al, u[d], fma(-3.0 * be, r[d], ar[d]));
+                    u[d] = fma(f.na3, r[d], vr[d]);
+                    ww[d] = fma(f.na6, u[d], fma(f.nb3, r[d], ar[d]));
                     const double g0 = tile[10 + d][e], g1 = tile[13 + d][e], g2 = tile[16 + d][e];
                     phil = fma(g0, r[d], fma(g1, u[d], fma(g2, ww[d], phil)));
                     phik = fma(gk[d], r[d], fma(gk[3 + d], u[d], fma(gk[6 + d], ww[d], phik)));
@@ -288,7 +290,7 @@ __global__ void __launch_bounds__(32 * W) adjoint_sym_kernel(SymArgs a, const do
                     gs[6 + d] = fma(mk, g2, -ml * gk[6 + d]);
                 }
                 double br[3], bv[3], ba[3];
-                bracket_from_phi(r, vr, ar, q2, al, be, fma(mk, phil, -ml * phik), gs, br, bv, ba);
+                bracket_from_phi(r, vr, ar, q2, al, be, f, fma(mk, phil, -ml * phik), gs, br, bv, ba);
 #pragma unroll
                 for (int d = 0; d < 3; ++d) {
                     ok[d] = fma(q3, br[d], ok[d]);
