@@ -22,28 +22,44 @@ __global__ void __launch_bounds__(256) predict_kernel(const double *__restrict__
                                                       const double *__restrict__ m, int n, double t,
                                                       double2 *__restrict__ jb64,
                                                       float *__restrict__ jf32, size_t npad,
-                                                      int mode)
+                                                      int mode, const int32_t *__restrict__ act, int n_act,
+                                                      int32_t *__restrict__ rows)
 {
     const size_t N = static_cast<size_t>(n);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const double d = t - ti[i];
-        Taylor p[3];
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
+        int i = p;  // row of particle p
+        if (n_act > 0) {
+            int lo = 0, hi = n_act;  // listed particles before p
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (act[mid] < p)
+                    lo = mid + 1;
+                else
+                    hi = mid;
+            }
+            const bool listed = lo < n_act && act[lo] == p;
+            i = listed ? lo : n_act + p - lo;
+            if (listed)
+                rows[lo] = lo;
+        }
+        const double d = t - ti[p];
+        Taylor e[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k)
-            p[k] = taylor(st[(F_X * 3 + k) * N + i], st[(F_V * 3 + k) * N + i],
-                          st[(F_A * 3 + k) * N + i], st[(F_J * 3 + k) * N + i],
-                          st[(F_S * 3 + k) * N + i], st[(F_C * 3 + k) * N + i], d);
-        const double mi = m[i];
+            e[k] = taylor(st[(F_X * 3 + k) * N + p], st[(F_V * 3 + k) * N + p],
+                          st[(F_A * 3 + k) * N + p], st[(F_J * 3 + k) * N + p],
+                          st[(F_S * 3 + k) * N + p], st[(F_C * 3 + k) * N + p], d);
+        const double mi = m[p];
         if (jb64) {
-            jb64[i] = make_double2(p[0].x, p[1].x);
-            jb64[N + i] = make_double2(p[2].x, mi);
-            jb64[2 * N + i] = make_double2(p[0].v, p[1].v);
-            jb64[3 * N + i] = make_double2(p[2].v, p[0].a);
-            jb64[4 * N + i] = make_double2(p[1].a, p[2].a);
+            jb64[i] = make_double2(e[0].x, e[1].x);
+            jb64[N + i] = make_double2(e[2].x, mi);
+            jb64[2 * N + i] = make_double2(e[0].v, e[1].v);
+            jb64[3 * N + i] = make_double2(e[2].v, e[0].a);
+            jb64[4 * N + i] = make_double2(e[1].a, e[2].a);
         }
         if (jf32 && mode == kModeEx) {
             // 20 rows: x, v, a (hi then lo per component group), m hi, m lo
-            const double q[9] = {p[0].x, p[1].x, p[2].x, p[0].v, p[1].v, p[2].v, p[0].a, p[1].a, p[2].a};
+            const double q[9] = {e[0].x, e[1].x, e[2].x, e[0].v, e[1].v, e[2].v, e[0].a, e[1].a, e[2].a};
 #pragma unroll
             for (int g = 0; g < 3; ++g)
 #pragma unroll
@@ -61,8 +77,8 @@ __global__ void __launch_bounds__(256) predict_kernel(const double *__restrict__
             float h[3], l[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                h[k] = nbk::to_float(p[k].x);
-                l[k] = drop_lo ? 0.0f : nbk::to_float(p[k].x - nbk::to_double(h[k]));
+                h[k] = nbk::to_float(e[k].x);
+                l[k] = drop_lo ? 0.0f : nbk::to_float(e[k].x - nbk::to_double(h[k]));
             }
             jf32[0 * npad + i] = h[0];
             jf32[1 * npad + i] = h[1];
@@ -73,8 +89,8 @@ __global__ void __launch_bounds__(256) predict_kernel(const double *__restrict__
             jf32[6 * npad + i] = l[2];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                jf32[(7 + k) * npad + i] = nbk::to_float(p[k].v);
-                jf32[(10 + k) * npad + i] = nbk::to_float(p[k].a);
+                jf32[(7 + k) * npad + i] = nbk::to_float(e[k].v);
+                jf32[(10 + k) * npad + i] = nbk::to_float(e[k].a);
             }
         }
     }
@@ -82,7 +98,7 @@ __global__ void __launch_bounds__(256) predict_kernel(const double *__restrict__
 
 }  // namespace
 
-cudaError_t nb_launch_predict(nb_ctx *c, double t)
+static cudaError_t launch_predict(nb_ctx *c, double t, const int32_t *act, int n_act, int32_t *out_rows)
 {
     const int n = static_cast<int>(c->n);
     const int block = 256;
@@ -91,7 +107,14 @@ cudaError_t nb_launch_predict(nb_ctx *c, double t)
     const int mode = c->cfg.precision == NB_EX ? kModeEx : (c->cfg.precision == NB_SP ? kModeSp : kModeMixed);
     predict_kernel<<<grid, block, 0, c->stream>>>(c->st, c->t, c->m, n, t, rows ? nullptr : c->jb64,
                                                   rows ? c->jf32 : nullptr,
-                                                  static_cast<size_t>(c->npad), mode);
+                                                  static_cast<size_t>(c->npad), mode, act, n_act, out_rows);
     c->launches += 1;
     return cudaGetLastError();
+}
+
+cudaError_t nb_launch_predict(nb_ctx *c, double t) { return launch_predict(c, t, nullptr, 0, nullptr); }
+
+cudaError_t nb_launch_predict_front(nb_ctx *c, double t, const int32_t *act, int n_act, int32_t *rows)
+{
+    return launch_predict(c, t, act, n_act, rows);
 }

@@ -595,11 +595,14 @@ int first_kind(int precision) { return nb_fp32_eval(precision) ? 0 : precision =
 // many), plus a fixed part per job and launch and the traffic of the slots.
 // Mixed: within 5 % of the measured times of the plans it chooses from 4096 to
 // 524288 particles; the next best plans lie within 2 % there.
-void nb_sym_plan_shape(const SymShape &kd, int kind, int64_t n, int sms, SymPlan &best)
+void nb_sym_plan_shape(const SymShape &kd, int kind, int64_t n, int sms, SymPlan &best,
+                       size_t max_bytes)
 {
     const int64_t T = (n + kd.tile - 1) / kd.tile, D = T / 2 + 1;
     const double slot = static_cast<double>(kd.bytes) * static_cast<double>(T * kd.tile);
-    const int64_t slots = std::max<int64_t>(2, static_cast<int64_t>(std::min(kSymSlotBytes, std::max(kSymMinBytes, kSymSlots * slot)) / slot));
+    const double budget = std::min(kSymSlotBytes, std::max(kSymMinBytes, kSymSlots * slot));
+    const int64_t slots = max_bytes ? static_cast<int64_t>(std::min(budget, static_cast<double>(max_bytes)) / slot)
+                                    : std::max<int64_t>(2, static_cast<int64_t>(budget / slot));
     const int subs = kd.tile / kd.threads;
     for (const int k : {1, 2, 4, 8})
         for (int parts = 1; parts <= subs; ++parts) {
@@ -631,11 +634,12 @@ void nb_sym_plan_shape(const SymShape &kd, int kind, int64_t n, int sms, SymPlan
         }
 }
 
-SymPlan nb_sym_plan(int precision, int64_t n, int sms)
+SymPlan nb_sym_plan(int precision, int64_t n, int sms, size_t max_bytes)
 {
     SymPlan best;
     for (int q = 0; q < 3; ++q)
-        nb_sym_plan_shape(kKinds[first_kind(precision) + q].shape, first_kind(precision) + q, n, sms, best);
+        nb_sym_plan_shape(kKinds[first_kind(precision) + q].shape, first_kind(precision) + q, n, sms, best,
+                          max_bytes);
     return best;
 }
 
@@ -652,7 +656,7 @@ cudaError_t nb_sym_smem_setup()
 }
 
 cudaError_t nb_launch_sym(int precision, const SymPlan &pl, const void *jb, size_t np, int n, double eps2,
-                          void *work, double *out, size_t ostride, cudaStream_t stream, int *launches)
+                          void *work, double *out, size_t ostride, bool add, cudaStream_t stream, int *launches)
 {
     const SymKind &kind = kKinds[pl.kind];
     const SymShape &kd = kind.shape;
@@ -681,7 +685,7 @@ cudaError_t nb_launch_sym(int precision, const SymPlan &pl, const void *jb, size
             using P = typename F::Part;
             fold_kernel<F><<<grid, 256, 0, stream>>>(static_cast<const P *>(a.pi), groups * pl.parts, upper,
                                                      static_cast<const P *>(a.pj), a.d0, a.d1, a.ns, pl.T,
-                                                     kd.tile, n, out, ostride, d0 == 0);
+                                                     kd.tile, n, out, ostride, d0 == 0 && !add);
         };
         if (precision == NB_FP64)
             fold(Fold64{});

@@ -271,14 +271,19 @@ nb_tiles nb_auto_tiles(const nb_ctx *c, int64_t n_act, const nb_tiles &req, int6
                        double *us = nullptr);
 cudaError_t nb_eval_smem_setup();
 // k_sym.cu
-SymPlan nb_sym_plan(int precision, int64_t n, int sms);
+// max_bytes: of partial sums (0: as many as a context's own plan may use)
+SymPlan nb_sym_plan(int precision, int64_t n, int sms, size_t max_bytes = 0);
 cudaError_t nb_sym_smem_setup();
 // jb, np: predicted particles and row stride; work: plan.bytes of device
-// memory, 256-byte aligned; out [9][ostride]; *launches counts kernels.
+// memory, 256-byte aligned; out [9][ostride], added to where `add`; *launches
+// counts kernels.
 cudaError_t nb_launch_sym(int precision, const SymPlan &plan, const void *jb, size_t np, int n, double eps2,
-                          void *work, double *out, size_t ostride, cudaStream_t stream, int *launches);
+                          void *work, double *out, size_t ostride, bool add, cudaStream_t stream, int *launches);
 // k_predict.cu
 cudaError_t nb_launch_predict(nb_ctx *c, double t);
+// The same into active-first order: rows [0, n_act) are the particles of the
+// ascending list act, the others follow in ascending order; rows[k] = k.
+cudaError_t nb_launch_predict_front(nb_ctx *c, double t, const int32_t *act, int n_act, int32_t *rows);
 // k_correct.cu
 cudaError_t nb_launch_correct(nb_ctx *c, double t1, int n_act);
 cudaError_t nb_launch_init_state(nb_ctx *c, int pass);

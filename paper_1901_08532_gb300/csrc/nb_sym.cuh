@@ -156,4 +156,4 @@ struct SymShape {
 };
 
 // k_sym.cu: best becomes the plan for this kernel where that is faster.
-void nb_sym_plan_shape(const SymShape &kd, int kind, int64_t n, int sms, SymPlan &best);
+void nb_sym_plan_shape(const SymShape &kd, int kind, int64_t n, int sms, SymPlan &best, size_t max_bytes = 0);
