@@ -66,11 +66,14 @@ def set_device_peaks(torch, dev):
     PEAK_FP32_TFLOPS = SM_COUNT * 128 * 2 * SM_MAX_MHZ * 1e6 / 1e12
     PEAK_FP64_TFLOPS = SM_COUNT * 2 * 2 * SM_MAX_MHZ * 1e6 / 1e12
     PEAK_FP32_OPS = SM_COUNT * 128 * SM_MAX_MHZ * 1e6
-# DRAM traffic of one mixed evaluation launch (the bench's own launch, one
-# ncu pass); valid only for the kernel source it was measured on (the sha256
-# prefix of csrc/k_eval.cu and csrc/nb_device.cuh).
-TRAFFIC = {"kernel_sha": "3b4746f198356227", "bytes_per_launch": 147.528960e6 + 70.369280e6,
-           "source": "ncu dram__bytes_read.sum + dram__bytes_write.sum, one pass on this launch"}
+# DRAM traffic of one mixed all-active evaluation (its pair and fold launches,
+# one ncu pass each); valid only for the kernel source it was measured on (the
+# sha256 prefix of TRAFFIC_FILES under csrc).
+TRAFFIC_FILES = ("k_sym.cu", "nb_sym.cuh", "nb_device.cuh")
+TRAFFIC = {"kernel_sha": "", "bytes_per_evaluation": None,
+           "source": "ncu dram__bytes_read.sum + dram__bytes_write.sum over the evaluation's launches"}
+# FP32-pipe operations per unordered pair in sym_mixed_kernel; per interaction half of them.
+SYM_OPS_PER_PAIR = 63
 WORKLOAD = "plummer_salpeter_N1048576_eps1e-4_shared_step_all_active"
 METRIC = "acc+jerk+snap interactions/s at N=2^20, mixed vs FP64 at rel err <= 1e-6"
 
@@ -323,7 +326,7 @@ class Clocks:
 
 def _kernel_sha():
     h = hashlib.sha256()
-    for name in ("k_eval.cu", "nb_device.cuh"):
+    for name in TRAFFIC_FILES:
         with open(os.path.join(ROOT, "paper_1901_08532_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -426,7 +429,7 @@ def run_ours(args):
     eval_s = sum(eval_ms) / len(eval_ms) / 1e3
     achieved = FLOPS_PER_INTERACTION * float(n) * (hi - lo) / eval_s / 1e12
     # the DRAM figure is of the whole-range launch; a rank's j-range launch is another workload
-    traffic = (TRAFFIC["bytes_per_launch"] if TRAFFIC["kernel_sha"] == _kernel_sha() and not split
+    traffic = (TRAFFIC["bytes_per_evaluation"] if TRAFFIC["kernel_sha"] == _kernel_sha() and not split
                else None)
     clocks = clk.summary()
     peaks = measure_peaks(nb, torch)
@@ -459,7 +462,7 @@ def run_ours(args):
                    "parallelism": (f"j-split x{world} (all-reduce of [9][N] FP64 partial sums per step)"
                                    if split else f"replicas x{world}" if world > 1 else "single GPU"),
                    "flops_per_interaction": FLOPS_PER_INTERACTION},
-        "roofline": {"bound": "alu", "kernel": "eval_mixed_kernel",
+        "roofline": {"bound": "alu", "kernel": "eval_mixed_kernel" if split else "sym_mixed_kernel",
                      "achieved": achieved, "peak": PEAK_FP32_TFLOPS, "unit": "TFLOP/s",
                      "frac": achieved / PEAK_FP32_TFLOPS, "traffic": traffic,
                      "peak_source": f"{SM_COUNT} SMs x 128 FP32 lanes x 2 flops x {SM_MAX_MHZ:g} MHz "
@@ -468,7 +471,12 @@ def run_ours(args):
                      "peak_measured_source": "nb_peak_probe: f32x2 FMA throughput "
                                              f"{peaks['fp32_fma_per_clk_per_sm']:.1f}/clk/SM x 2 flops x "
                                              f"{SM_COUNT} SMs x {SM_MAX_MHZ:g} MHz",
-                     "eval_ms_mean": 1e3 * eval_s},
+                     "eval_ms_mean": 1e3 * eval_s}
+        | ({} if split else {
+            "note": "achieved counts 78 flop for each of the N^2 interactions; the kernel takes each "
+                    "unordered pair once",
+            "fp32_pipe_ops_per_interaction": SYM_OPS_PER_PAIR / 2,
+            "fp32_pipe_frac": SYM_OPS_PER_PAIR / 2 * float(n) * n / eval_s / PEAK_FP32_OPS}),
         "peaks": {k: peaks[k] for k in ("fp32_fma_per_clk_per_sm", "fp64_fma_per_clk_per_sm",
                                         "fp32_tflops_at_max_clock", "fp64_tflops_at_max_clock")} | {
             "per_clk_per_sm": {k: round(v["ops_per_clk_per_sm"], 2) for k, v in peaks["kinds"].items()},
@@ -660,7 +668,8 @@ def end_to_end(nb, np, torch, ctx, n, stream, steps, split=None):
 
 def profile_eval(args):
     """Evaluation launches only: Plummer/Salpeter N = --n, --n-act seeded
-    active particles, --reps launches (for ncu; prints per-launch times)."""
+    active particles (all of them from --n on), --reps launches (for ncu;
+    prints per-launch times)."""
     import numpy as np
     import torch
 
@@ -674,7 +683,9 @@ def profile_eval(args):
     ctx = nb.NBody(m, x, v, EPS, precision=prec, stream=stream, start_forces=False)
     ctx.set_state({"a": a})
     ctx.predict(0.0)
-    act = torch.from_numpy(ni.active_subset(args.n, args.n_act, 7)).cuda()
+    args.n_act = min(args.n_act, args.n)
+    act = (None if args.n_act == args.n
+           else torch.from_numpy(ni.active_subset(args.n, args.n_act, 7)).cuda())
     times = []
     for _ in range(args.reps):
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -860,14 +871,13 @@ def integrate_run(nb, np, torch, n, prec_name, t_end=1.0 / 16, step_noise=0.0):
     E1 = sum(ctx.energy())
     ctx.close()
     hist = np.bincount(np.floor(np.log2(np.maximum(ln, 1))).astype(int))
-    flops = FLOPS_PER_INTERACTION * float(n) * n / full_s / 1e12
-    peak = PEAK_FP64_TFLOPS if prec == nb.NB_FP64 else PEAK_FP32_TFLOPS
-    n_fp32_ops = {nb.NB_EX: EX_OPS_PER_INTERACTION}.get(prec)
+    # operations of the bounding pipe per unordered pair (each pair is taken once)
+    pair_ops = {nb.NB_FP64: 60, nb.NB_EX: 608}.get(prec, SYM_OPS_PER_PAIR)
+    pipe = PEAK_FP64_TFLOPS / 2 * 1e12 if prec == nb.NB_FP64 else PEAK_FP32_OPS
     return {"workload": f"plummer_N{n}_eps1e-4_{prec_name}" + (f"_noise{step_noise:g}" if step_noise else ""),
             "full_eval_s": full_s,
             "full_eval_interactions_per_s": float(n) * n / full_s,
-            "full_eval_frac_of_peak": (flops / peak if n_fp32_ops is None else
-                                       n_fp32_ops * float(n) * n / full_s / PEAK_FP32_OPS),
+            "full_eval_frac_of_pipe": pair_ops / 2 * float(n) * n / full_s / pipe,
             "integration_t_end": t_end, "block_steps": steps,
             "integration_s": el, "us_per_block_step": 1e6 * el / max(steps, 1),
             "integration_interactions": i1 - i0,
