@@ -22,8 +22,9 @@
  *     caller keeps ownership.  Vectors are [n][3] row-major doubles.
  *   - Device pointers passed in are borrowed for the call only and must be
  *     device memory of the context's device.
- *   - The context owns all of its device memory (allocated in nb_init,
- *     released in nb_free) and runs all work on the stream given in
+ *   - The context owns all of its device memory (allocated in nb_init, the
+ *     scratch for partial sums and samples by the first call that needs it,
+ *     never under stream capture; released in nb_free) and runs all work on the stream given in
  *     nb_config.stream (a cudaStream_t; NULL = the legacy default stream).
  *     Entry points that return host data synchronise that stream.
  *   - Softened gravity with G = 1: pair term from particle j on particle i

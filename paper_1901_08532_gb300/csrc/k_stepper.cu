@@ -300,8 +300,6 @@ cudaError_t launch_stepper(nb_ctx *c, StepArgs &a, int grid_max)
 
 }  // namespace
 
-int nb_stepper_small() { return kStepSmall; }
-
 // One launch of the device-resident stepper; reports what it did in *r
 // (synchronises the stream).  reason 1 leaves the next active set in
 // c->act_next.

@@ -298,7 +298,6 @@ cudaError_t nb_launch_iota(nb_ctx *c, int n, int32_t *dst);
 // nb_api.cu: message returned by nb_last_error(NULL) on this thread
 void nb_set_thread_error(const char *msg);
 // k_stepper.cu
-int nb_stepper_small();
 struct StepperResult {
     int64_t steps, act_sum;  // block steps taken and the active particles summed over them
     int reason;              // 0: t_end reached, 1: next active set too large, 2: error flag
