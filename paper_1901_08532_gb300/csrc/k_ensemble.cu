@@ -782,7 +782,8 @@ __global__ void __launch_bounds__(kEnsThreads, 1) ensemble_kernel(EnsArgs a)
         for (;;) {
             const int par = static_cast<int>(steps & 1);
             // schedule, one pass: the slice's earliest t_i + dt_i and how many
-            // particles reach it; a small set is listed in shared memory
+            // particles reach it; a small set is listed in shared memory (an
+            // ensemble starts at t = 0, so the bits order like the times)
             unsigned long long mt = ~0ull;
             int ct = 0;
             for (int i = c0; i < c1; ++i) {

@@ -4,8 +4,8 @@
 // dyadic rationals, so the sums and the equality test are exact.
 //
 // Three small launches over the 16 bytes/particle of (t, dt):
-//   1. min-reduction (positive doubles order like their bit patterns, so an
-//      integer atomicMin on the bits is exact),
+//   1. min-reduction (integer atomicMin on keys that order like the times,
+//      negative ones included, so it is exact),
 //   2. per-block counts of due particles,
 //   3. ordered compaction: each block adds the counts of the blocks before
 //      it, scans its own flags and writes indices; the last block stores
@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(kThreads) tmin_kernel(const double *t, const d
 {
     unsigned long long best = ~0ull;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(t[i] + dt[i]));
+        const unsigned long long b = nbk::time_key(t[i] + dt[i]);
         best = b < best ? b : best;
     }
     for (int off = 16; off > 0; off >>= 1) {
@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(kThreads) tmin_kernel(const double *t, const d
         best = o < best ? o : best;
     }
     if ((threadIdx.x & 31) == 0)
-        atomicMin(&ctl->tnext_bits, best);
+        atomicMin(&ctl->tnext_key, best);
 }
 
 __device__ __forceinline__ bool due(const double *t, const double *dt, int i, double tn)
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(kThreads) count_kernel(const double *t, const 
                                                          const nb_ctl *ctl, int32_t *blk)
 {
     __shared__ int s_cnt[kThreads / 32];
-    const double tn = __longlong_as_double(static_cast<long long>(ctl->tnext_bits));
+    const double tn = nbk::time_of(ctl->tnext_key);
     const int base = blockIdx.x * kPerBlock + threadIdx.x * kPerThread;
     int c = 0;
 #pragma unroll
@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kThreads) compact_kernel(const double *t, cons
 {
     __shared__ int s_w[kThreads / 32];
     __shared__ int s_prefix;
-    const double tn = __longlong_as_double(static_cast<long long>(ctl->tnext_bits));
+    const double tn = nbk::time_of(ctl->tnext_key);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
     // counts of all earlier blocks
@@ -130,7 +130,7 @@ __global__ void iota_kernel(int32_t *act, int n)
 cudaError_t nb_launch_schedule(nb_ctx *c)
 {
     const int n = static_cast<int>(c->n);
-    cudaError_t e = cudaMemsetAsync(&c->ctl->tnext_bits, 0xff, sizeof(unsigned long long), c->stream);
+    cudaError_t e = cudaMemsetAsync(&c->ctl->tnext_key, 0xff, sizeof(unsigned long long), c->stream);
     if (e != cudaSuccess)
         return e;
     int g1 = (n + kThreads - 1) / kThreads;

@@ -73,7 +73,7 @@ struct StepArgs {
     const double *m;
     double eps2, eta, dt_min, dt_max, dt_shared, t_end, noise;
     int drop_lo;        // single-precision control: positions without their low part
-    unsigned long long *bmin;  // [B] per-block earliest t_i + dt_i, as bits
+    unsigned long long *bmin;  // [B] per-block earliest t_i + dt_i, as time_key()
     int *bcnt;          // [B] particles reaching it
     int *cand;          // [B][kStepSmall] their indices, ascending
     double *part;       // [kStepSmall][9][B] partial sums
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(T) step_kernel(StepArgs a)
         unsigned long long mt = ~0ull;
         int ct = 0;
         for (int i = c0; i < c1; ++i) {
-            const unsigned long long tt = static_cast<unsigned long long>(__double_as_longlong(a.t[i] + a.dt[i]));
+            const unsigned long long tt = time_key(a.t[i] + a.dt[i]);
             if (tt < mt) {
                 mt = tt;
                 ct = 1;
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(T) step_kernel(StepArgs a)
         if (mine > 0 && tot_b <= kStepSmall) {
             int pos = ex;
             for (int i = c0; i < c1; ++i)
-                if (static_cast<unsigned long long>(__double_as_longlong(a.t[i] + a.dt[i])) == mb)
+                if (time_key(a.t[i] + a.dt[i]) == mb)
                     a.cand[bk * kStepSmall + pos++] = i;
         }
         if (tid == 0) {
@@ -135,22 +135,22 @@ __global__ void __launch_bounds__(T) step_kernel(StepArgs a)
         grid.sync();
         // the same decision in every block: thread tid looks at the blocks
         // kQ tid .. kQ tid + kQ - 1
-        unsigned long long bm[kQ], mn_bits = ~0ull;
+        unsigned long long bm[kQ], mn_key = ~0ull;
         int bc[kQ];
 #pragma unroll
         for (int e = 0; e < kQ; ++e) {
             const int q = tid * kQ + e;
             bm[e] = q < B ? __ldcg(&a.bmin[q]) : ~0ull;
             bc[e] = q < B ? __ldcg(&a.bcnt[q]) : 0;
-            mn_bits = bm[e] < mn_bits ? bm[e] : mn_bits;
+            mn_key = bm[e] < mn_key ? bm[e] : mn_key;
         }
         const int err = *reinterpret_cast<volatile int *>(&a.ctl->err);
-        mn_bits = block_min_u64(mn_bits, red_u);
-        const double mn = __longlong_as_double(static_cast<long long>(mn_bits));
+        mn_key = block_min_u64(mn_key, red_u);
+        const double mn = time_of(mn_key);
         int c = 0;
 #pragma unroll
         for (int e = 0; e < kQ; ++e)
-            c += bm[e] == mn_bits ? bc[e] : 0;
+            c += bm[e] == mn_key ? bc[e] : 0;
         int total = 0;
         int pos = block_scan_excl(c, red_i, &total);
         if (err) {
@@ -169,13 +169,13 @@ __global__ void __launch_bounds__(T) step_kernel(StepArgs a)
             for (int e = 0, q = pos; e < kQ; ++e) {
                 if (tid * kQ + e == bk)
                     red_i[0] = q;
-                q += bm[e] == mn_bits ? bc[e] : 0;
+                q += bm[e] == mn_key ? bc[e] : 0;
             }
             __syncthreads();
-            if (mine > 0 && mb == mn_bits) {
+            if (mine > 0 && mb == mn_key) {
                 int at = red_i[0] + ex;
                 for (int i = c0; i < c1; ++i)
-                    if (static_cast<unsigned long long>(__double_as_longlong(a.t[i] + a.dt[i])) == mb)
+                    if (time_key(a.t[i] + a.dt[i]) == mb)
                         a.act_next[at++] = i;
             }
             next_t = mn;
@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(T) step_kernel(StepArgs a)
         // active list, ascending: blocks in order, each block's list in order
 #pragma unroll
         for (int e = 0; e < kQ; ++e)
-            if (bm[e] == mn_bits)
+            if (bm[e] == mn_key)
                 for (int u = 0; u < bc[e]; ++u)
                     s_act[pos++] = (tid * kQ + e) * kStepSmall + u;
         __syncthreads();

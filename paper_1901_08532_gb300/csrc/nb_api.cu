@@ -296,7 +296,7 @@ nb_status schedule(nb_ctx *c, double *tn, int64_t *n_act)
     nb_status s = sync_ctl(c);
     if (s != NB_OK)
         return s;
-    unsigned long long b = c->ctl_h->tnext_bits;
+    const unsigned long long b = nbk::time_key_bits(c->ctl_h->tnext_key);
     double t;
     std::memcpy(&t, &b, sizeof t);
     *tn = t;

@@ -19,7 +19,8 @@ struct StateView {
 // Bytes per j-record in shared memory: FP64 5 x 16, mixed 13 x 4, EX 20 x 4.
 __host__ __device__ constexpr int rec_bytes(int pr) { return pr == 0 ? 80 : (pr == 1 ? NCF * 4 : NCX * 4); }
 
-// Block minimum of 64-bit values (non-negative doubles order like their bits).
+// Block minimum of 64-bit values (times as time_key(), or as their bits where
+// none is negative).
 __device__ __forceinline__ unsigned long long block_min_u64(unsigned long long v, unsigned long long *red)
 {
     for (int o = 16; o > 0; o >>= 1) {

@@ -34,7 +34,7 @@ inline int nb_jrows(int precision)
 }
 
 struct nb_ctl {                      // small device control block
-    unsigned long long tnext_bits;   // min over i of (t_i + dt_i), as bits
+    unsigned long long tnext_key;    // min over i of (t_i + dt_i), as time_key()
     int32_t n_act;                   // active count from the scheduler
     int32_t err;                     // bit flags, see NB_ERR_*
     int64_t floor_hits;              // steps clamped at dt_min
@@ -117,6 +117,24 @@ struct nb_ctx {
 // --------------------------------------------------------- device helpers
 
 namespace nbk {
+
+// Key of a time that orders, as an unsigned integer, like the time itself (the
+// bits of a double alone do so from 0 on only; a state may hold negative
+// times), on the integer pipe; one to one.  ~0 is the key of a NaN, behind
+// every time.
+__device__ __forceinline__ unsigned long long time_key(double t)
+{
+    const long long b = __double_as_longlong(t);
+    return static_cast<unsigned long long>(b) ^ (static_cast<unsigned long long>(b >> 63) | 1ull << 63);
+}
+__host__ __device__ constexpr unsigned long long time_key_bits(unsigned long long key)
+{
+    return key ^ (key >> 63 ? 1ull << 63 : ~0ull);
+}
+__device__ __forceinline__ double time_of(unsigned long long key)
+{
+    return __longlong_as_double(static_cast<long long>(time_key_bits(key)));
+}
 
 __device__ __forceinline__ unsigned long long globaltimer_ns()
 {
