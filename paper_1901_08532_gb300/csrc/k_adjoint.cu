@@ -440,7 +440,7 @@ nb_status nb_pairs_fp64(int64_t n, const double *m, const double *x, const doubl
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)
-        e = pw.sym ? nb_launch_sym(NB_FP64, pw.plan, rec, static_cast<size_t>(nn), nn, eps * eps, w + pw.slots, sums,
+        e = pw.sym ? nb_launch_sym(NB_FP64, pw.plan, rec, static_cast<size_t>(nn), nn, eps * eps, false, w + pw.slots, sums,
                                    static_cast<size_t>(nn), false, s, &launches)
                    : nb_launch_eval_fp64_rows(rec, nn, iota, sums, eps * eps, ctl, s, sms);
     if (e == cudaSuccess) {

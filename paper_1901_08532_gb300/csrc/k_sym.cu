@@ -4,7 +4,8 @@
 // and beta.  Swapping i and j negates r, v and a, keeps alpha and beta, and
 // so negates u and w: the terms on j are (-m_i / m_j) times those on i.  Per
 // unordered pair the mixed formula takes 63 FP32-pipe operations instead of
-// 2 x 53 (FP64 60 instead of 100, EX 608 instead of 992).
+// 2 x 53 (FP64 60 instead of 100, EX 608 instead of 992; one product more with
+// masses above 1).
 //
 // Work split.  The particles form T tiles of B; a job (b, d) is the pairs of
 // tile b with tile (b + d) mod T, and d = 0 .. T/2 covers every unordered pair
@@ -60,9 +61,44 @@ constexpr int kMixedWarps = 4;
 constexpr int kMixedThreads = 32 * kMixedWarps;
 __host__ __device__ constexpr int mixed_tile(int kp) { return kMixedThreads * 2 * kp; }
 
+// mu = m_j q^3 and nu = -m_i q^3.  q^3 by itself leaves the FP32 range from
+// separations of 2^42 on (and the low word of a double word from 2^26 on); where
+// no mass is above 1 (LIGHT), m q^3 is no larger than it and leaves the range with it or
+// before, so it may be formed once for both.  Larger masses, such as G m in metres
+// or centimetres, come in before the second power of q, as in the ordinary
+// kernels: one product more, 3.6 % (mixed) and 1.5 % (EX) of the time (524288
+// particles mixed 296 / 306 ms, 40000 EX 15.0 / 15.2 ms).
+template <bool LIGHT>
+__device__ __forceinline__ void mass_factors(float2 q, float2 q2, float2 mj, float2 nmi, float2 &mu, float2 &nu)
+{
+    if constexpr (LIGHT) {
+        const float2 q3 = mul2(q, q2);
+        mu = mul2(mj, q3);
+        nu = mul2(nmi, q3);
+    } else {
+        mu = mul2(mul2(mj, q), q2);
+        nu = mul2(mul2(nmi, q), q2);
+    }
+}
+template <bool LIGHT>
+__device__ __forceinline__ void mass_factors(const ff::FF<float2> &q, const ff::FF<float2> &q2,
+                                             const ff::FF<float2> &mj, const ff::FF<float2> &nmi,
+                                             ff::FF<float2> &mu, ff::FF<float2> &nu)
+{
+    if constexpr (LIGHT) {
+        const ff::FF<float2> q3 = ff::mul(q, q2);
+        mu = ff::mul(mj, q3);
+        nu = ff::mul(nmi, q3);
+    } else {
+        mu = ff::mul(ff::mul(mj, q), q2);
+        nu = ff::mul(ff::mul(nmi, q), q2);
+    }
+}
+
 // Both directions of the pairs of two i-particles (the lanes of the packed
 // values) with one j: pi += terms on i, pj += terms on j.  ni are the negated
 // i-values, nmi the negated masses, c the 13 j-values.
+template <bool LIGHT>
 __device__ __forceinline__ void pair_mixed_sym(const float (&c)[NCF], const float2 (&ni)[12], float2 nmi,
                                                float2 eps2, float2 (&pi)[9], float2 (&pj)[9])
 {
@@ -76,8 +112,8 @@ __device__ __forceinline__ void pair_mixed_sym(const float (&c)[NCF], const floa
     const float2 sv = fma2(dx, dax, fma2(dy, day, fma2(dz, daz, fma2(dvx, dvx, fma2(dvy, dvy, mul2(dvz, dvz))))));
     const float2 q = make_float2(rsqrt_est(r2.x), rsqrt_est(r2.y));
     const float2 q2 = make_float2(rcp_est(r2.x), rcp_est(r2.y));
-    const float2 q3 = mul2(q, q2);
-    const float2 mu = mul2(f2(c[3]), q3), nu = mul2(nmi, q3);
+    float2 mu, nu;
+    mass_factors<LIGHT>(q, q2, f2(c[3]), nmi, mu, nu);
     const float2 al = mul2(rv, q2);
     const float2 be = fma2(al, al, mul2(sv, q2));
     const float2 na3 = mul2(al, f2(-3.0f)), na6 = mul2(al, f2(-6.0f)), nb3 = mul2(be, f2(-3.0f));
@@ -122,7 +158,7 @@ __device__ __forceinline__ void load_tile_mixed(const SymArgs &a, float *dst, in
 // 4096 51 -> 39 us, 8192 150 -> 111, 20011 744 -> 500, 65536 7.26 -> 4.80 ms,
 // 131072 28.6 -> 18.7 ms, 2^20 1.813 -> 1.178 s.  Below about 3500 particles the ordinary kernels
 // are faster (3000: 34 us against 39).
-template <int KP>
+template <int KP, bool LIGHT>
 __global__ void __launch_bounds__(kMixedThreads, 2) sym_mixed_kernel(SymArgs a)
 {
     constexpr int W = kMixedWarps, TH = kMixedThreads, B = mixed_tile(KP);
@@ -179,7 +215,7 @@ __global__ void __launch_bounds__(kMixedThreads, 2) sym_mixed_kernel(SymArgs a)
                         c[r] = sj[r * TH];
 #pragma unroll
                     for (int p = 0; p < KP; ++p)
-                        pair_mixed_sym(c, ni[p], nmi[p], eps2, pi[p], pj);
+                        pair_mixed_sym<LIGHT>(c, ni[p], nmi[p], eps2, pi[p], pj);
 #pragma unroll
                     for (int q = 0; q < 9; ++q) {
                         pj[q].x = __shfl_sync(0xffffffffu, pj[q].x, lane + 1);
@@ -248,6 +284,7 @@ __host__ __device__ constexpr int ex_tile(int w) { return 64 * w; }
 // Both directions of the pairs of two i-particles with one j in double words
 // (pair_ex with the powers of q shared): ni the negated i-values, nmi the
 // negated masses.
+template <bool LIGHT>
 __device__ __forceinline__ void pair_ex_sym(const float2 (&c)[NCX], const ExI<float2> &ni,
                                             const ff::FF<float2> &nmi, const ff::FF<float2> &eps2,
                                             ff::FF<float2> (&pi)[9], ff::FF<float2> (&pj)[9])
@@ -266,8 +303,8 @@ __device__ __forceinline__ void pair_ex_sym(const float2 (&c)[NCX], const ExI<fl
                  ff::mad(dv[0], dv[0], ff::mad(dv[1], dv[1], ff::sqr(dv[2]))))));
     const F q = ff::rsqrt(R, rsqrt_est_v(R.h));
     const F q2 = ff::sqr(q);
-    const F q3 = ff::mul(q, q2);
-    const F mu = ff::mul(F{c[18], c[19]}, q3), nu = ff::mul(nmi, q3);
+    F mu, nu;
+    mass_factors<LIGHT>(q, q2, F{c[18], c[19]}, nmi, mu, nu);
     const F al = ff::mul(rv, q2);
     const F be = ff::mad(al, al, ff::mul(sv, q2));
     const float2 m3 = f2(-3.0f), two = f2(2.0f);
@@ -294,7 +331,7 @@ __device__ __forceinline__ void pair_ex_sym(const float2 (&c)[NCX], const ExI<fl
 // All particles, ordinary kernel -> this one: 2000 81 -> 72 us, 4096 268 -> 207,
 // 16384 3.84 -> 2.58 ms, 40000 23.7 -> 15.0 ms (1.07e11 interactions/s).  Below
 // about 1800 particles the ordinary kernel is faster.
-template <int W>
+template <int W, bool LIGHT>
 __global__ void __launch_bounds__(32 * W, 8 / W) sym_ex_kernel(SymArgs a)
 {
     using F = ff::FF<float2>;
@@ -367,7 +404,7 @@ __global__ void __launch_bounds__(32 * W, 8 / W) sym_ex_kernel(SymArgs a)
 #pragma unroll
                 for (int r = 0; r < NCX; ++r)
                     c[r] = f2(sj[r * TH]);
-                pair_ex_sym(c, ni, nmi, eps2, pi, pj);
+                pair_ex_sym<LIGHT>(c, ni, nmi, eps2, pi, pj);
 #pragma unroll
                 for (int q = 0; q < 9; ++q) {
                     pj[q].h.x = __shfl_sync(0xffffffffu, pj[q].h.x, lane + 1);
@@ -568,21 +605,21 @@ constexpr size_t mixed_smem(int kp) { return sizeof(float) * kMixedThreads * (2 
 constexpr size_t ex_smem(int w) { return sizeof(float) * 32 * w * (2 * NCX + 18 + 36); }
 
 struct SymKind {
-    void (*kernel)(SymArgs);
+    void (*light)(SymArgs), (*heavy)(SymArgs);  // no mass above 1; any masses
     size_t smem;
     SymShape shape;
 };
 
 const SymKind kKinds[] = {
-    {sym_mixed_kernel<3>, mixed_smem(3), {mixed_tile(3), kMixedThreads, 72, 3170.0, 1.12}},
-    {sym_mixed_kernel<2>, mixed_smem(2), {mixed_tile(2), kMixedThreads, 72, 2750.0, 1.12}},
-    {sym_mixed_kernel<1>, mixed_smem(1), {mixed_tile(1), kMixedThreads, 72, 2200.0, 1.12}},
-    {sym_ex_kernel<4>, ex_smem(4), {ex_tile(4), 128, 72, 360.0, 1.3}},
-    {sym_ex_kernel<2>, ex_smem(2), {ex_tile(2), 64, 72, 355.0, 2.6}},
-    {sym_ex_kernel<1>, ex_smem(1), {ex_tile(1), 32, 72, 345.0, 5.2}},
-    {sym_fp64_kernel<4>, 0, {128, 128, 72, 60.0, 1.05}},
-    {sym_fp64_kernel<2>, 0, {64, 64, 72, 59.5, 2.1}},
-    {sym_fp64_kernel<1>, 0, {32, 32, 72, 58.5, 4.2}},
+    {sym_mixed_kernel<3, true>, sym_mixed_kernel<3, false>, mixed_smem(3), {mixed_tile(3), kMixedThreads, 72, 3170.0, 1.12}},
+    {sym_mixed_kernel<2, true>, sym_mixed_kernel<2, false>, mixed_smem(2), {mixed_tile(2), kMixedThreads, 72, 2750.0, 1.12}},
+    {sym_mixed_kernel<1, true>, sym_mixed_kernel<1, false>, mixed_smem(1), {mixed_tile(1), kMixedThreads, 72, 2200.0, 1.12}},
+    {sym_ex_kernel<4, true>, sym_ex_kernel<4, false>, ex_smem(4), {ex_tile(4), 128, 72, 360.0, 1.3}},
+    {sym_ex_kernel<2, true>, sym_ex_kernel<2, false>, ex_smem(2), {ex_tile(2), 64, 72, 355.0, 2.6}},
+    {sym_ex_kernel<1, true>, sym_ex_kernel<1, false>, ex_smem(1), {ex_tile(1), 32, 72, 345.0, 5.2}},
+    {sym_fp64_kernel<4>, sym_fp64_kernel<4>, 0, {128, 128, 72, 60.0, 1.05}},
+    {sym_fp64_kernel<2>, sym_fp64_kernel<2>, 0, {64, 64, 72, 59.5, 2.1}},
+    {sym_fp64_kernel<1>, sym_fp64_kernel<1>, 0, {32, 32, 72, 58.5, 4.2}},
 };
 
 // Kinds of a precision: [first, first + 3).
@@ -646,8 +683,10 @@ SymPlan nb_sym_plan(int precision, int64_t n, int sms, size_t max_bytes)
 cudaError_t nb_sym_smem_setup()
 {
     for (const SymKind &kd : kKinds)
-        if (kd.smem > 0) {
-            const cudaError_t e = cudaFuncSetAttribute(kd.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        for (auto kernel : {kd.light, kd.heavy}) {
+            if (kd.smem == 0)
+                continue;
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                        static_cast<int>(kd.smem));
             if (e != cudaSuccess)
                 return e;
@@ -656,7 +695,8 @@ cudaError_t nb_sym_smem_setup()
 }
 
 cudaError_t nb_launch_sym(int precision, const SymPlan &pl, const void *jb, size_t np, int n, double eps2,
-                          void *work, double *out, size_t ostride, bool add, cudaStream_t stream, int *launches)
+                          bool light, void *work, double *out, size_t ostride, bool add, cudaStream_t stream,
+                          int *launches)
 {
     const SymKind &kind = kKinds[pl.kind];
     const SymShape &kd = kind.shape;
@@ -678,7 +718,7 @@ cudaError_t nb_launch_sym(int precision, const SymPlan &pl, const void *jb, size
         const int64_t jobs = sym_jobs(pl.T, a.d0, a.d1, pl.k);
         const int groups = (a.d1 - a.d0 + pl.k - 1) / pl.k;
         const int upper = static_cast<int>(jobs / pl.T) * pl.parts;  // i-slots of the upper half of the tiles
-        kind.kernel<<<static_cast<unsigned>(jobs * pl.parts), kd.threads, kind.smem, stream>>>(a);
+        (light ? kind.light : kind.heavy)<<<static_cast<unsigned>(jobs * pl.parts), kd.threads, kind.smem, stream>>>(a);
         const dim3 grid((n + 255) / 256, 9);
         auto fold = [&](auto f) {
             using F = decltype(f);

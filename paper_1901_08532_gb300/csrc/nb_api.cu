@@ -149,7 +149,7 @@ cudaError_t launch_pairs(nb_ctx *c, const SymPlan &plan, int64_t n, double *out,
     int launches = 0;
     const cudaError_t e =
         nb_launch_sym(c->cfg.precision, plan, rows ? static_cast<const void *>(c->jf32) : c->jb64,
-                      static_cast<size_t>(rows ? c->npad : c->n), static_cast<int>(n), c->eps * c->eps, c->sym_work,
+                      static_cast<size_t>(rows ? c->npad : c->n), static_cast<int>(n), c->eps * c->eps, c->light, c->sym_work,
                       out, static_cast<size_t>(c->n), add, c->stream, &launches);
     c->launches += launches;
     return e;
@@ -503,6 +503,7 @@ nb_status nb_init(nb_ctx **out, int64_t n, const double *m, const double *x, con
     c->cfg = cf;
     c->n = n;
     c->eps = eps;
+    c->light = *std::max_element(m, m + n) <= 1.0;
     c->stream = static_cast<cudaStream_t>(cf.stream);
     auto bail = [&](nb_status s) {
         g_init_err = c->err;

@@ -83,6 +83,7 @@ struct nb_ctx {
     std::vector<void *> outgrown;  // earlier, smaller blocks of part and tile_cnt
     SymPlan sym_plan;          // evaluation of all particles, each pair once
     bool sym_use = false;
+    bool light = false;        // no mass is above 1
     void *sym_work = nullptr;  // its partial sums
     int32_t *blk = nullptr;    // scheduler block counts
     double *red = nullptr;     // reduction scratch
@@ -292,11 +293,12 @@ cudaError_t nb_eval_smem_setup();
 // max_bytes: of partial sums (0: as many as a context's own plan may use)
 SymPlan nb_sym_plan(int precision, int64_t n, int sms, size_t max_bytes = 0);
 cudaError_t nb_sym_smem_setup();
-// jb, np: predicted particles and row stride; work: plan.bytes of device
-// memory, 256-byte aligned; out [9][ostride], added to where `add`; *launches
-// counts kernels.
+// jb, np: predicted particles and row stride; light: no mass is above 1 (FP64: of
+// no effect); work: plan.bytes of device memory, 256-byte aligned; out
+// [9][ostride], added to where `add`; *launches counts kernels.
 cudaError_t nb_launch_sym(int precision, const SymPlan &plan, const void *jb, size_t np, int n, double eps2,
-                          void *work, double *out, size_t ostride, bool add, cudaStream_t stream, int *launches);
+                          bool light, void *work, double *out, size_t ostride, bool add, cudaStream_t stream,
+                          int *launches);
 // k_predict.cu
 cudaError_t nb_launch_predict(nb_ctx *c, double t);
 // The same into active-first order: rows [0, n_act) are the particles of the
