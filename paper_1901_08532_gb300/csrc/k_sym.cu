@@ -326,10 +326,11 @@ __device__ __forceinline__ void pair_ex_sym(const float2 (&c)[NCX], const ExI<fl
 
 // Bound by the FP32 pipe like the ordinary EX kernel; eight warps of 238
 // registers fill an SM, and the tile shrinks with W for small systems.
-// Double-word sums run over at most 64 terms in each half of a packed value, as
-// in the ordinary kernel; its RMS error is 0.95-1.0 of that kernel's.
+// Double-word sums run over at most 64 terms in each half of a packed value and
+// go to FP64 after at most 512, as in the ordinary kernel; its RMS error is 0.95-1.0
+// of that kernel's.
 // All particles, ordinary kernel -> this one: 2000 81 -> 72 us, 4096 268 -> 207,
-// 16384 3.84 -> 2.58 ms, 40000 23.7 -> 15.0 ms (1.07e11 interactions/s).  Below
+// 16384 3.84 -> 2.55 ms, 40000 23.7 -> 14.7 ms (1.08e11 interactions/s).  Below
 // about 1800 particles the ordinary kernel is faster.
 template <int W, bool LIGHT>
 __global__ void __launch_bounds__(32 * W, 8 / W) sym_ex_kernel(SymArgs a)
@@ -340,6 +341,7 @@ __global__ void __launch_bounds__(32 * W, 8 / W) sym_ex_kernel(SymArgs a)
     float *tile = sm;                 // [2][NCX][TH]
     float *jacc = sm + 2 * NCX * TH;  // [18][TH]: high parts of the 9 sums, then low parts
     float *iacc = jacc + 18 * TH;     // [2][18][TH]
+    double *itot = reinterpret_cast<double *>(iacc + 36 * TH);  // [2][9][TH]
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const SymJob<B, TH> job(a);
     const float *jf = static_cast<const float *>(a.jb);
@@ -365,8 +367,10 @@ __global__ void __launch_bounds__(32 * W, 8 / W) sym_ex_kernel(SymArgs a)
         pi[q] = {f2(0.0f), f2(0.0f)};
     for (int q = 0; q < 36; ++q)
         iacc[q * TH + tid] = 0.0f;
-    for (int q = 0; q < 18; ++q)
+    for (int q = 0; q < 18; ++q) {
         jacc[q * TH + tid] = 0.0f;
+        itot[q * TH + tid] = 0.0;
+    }
 
     auto load = [&](int it) {
         float *dst = tile + (it & 1) * NCX * TH;
@@ -383,6 +387,7 @@ __global__ void __launch_bounds__(32 * W, 8 / W) sym_ex_kernel(SymArgs a)
         h[0] = s.h;
         h[ld] = s.l;
     };
+    auto wide = [](const float *h, int ld) { return to_double(h[0]) + to_double(h[ld]); };
     if (job.nit > 0)
         load(0);
     for (int it = 0; it < job.nit; ++it) {
@@ -429,21 +434,29 @@ __global__ void __launch_bounds__(32 * W, 8 / W) sym_ex_kernel(SymArgs a)
                 }
             __syncthreads();
         }
-        float2 *out = static_cast<float2 *>(a.pj) + job.jslot(a, it) + tid;
+        double *out = static_cast<double *>(a.pj) + job.jslot(a, it) + tid;
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
             if (job.offset(it) > 0)
-                out[q * a.ns] = make_float2(jacc[q * TH + tid], jacc[(9 + q) * TH + tid]);
+                out[q * a.ns] = wide(jacc + q * TH + tid, 9 * TH);
             jacc[q * TH + tid] = 0.0f;
             jacc[(9 + q) * TH + tid] = 0.0f;
         }
+        // i-sums over at most 512 j in double words, like the ordinary kernel's
+        // tiles, then FP64
+        if ((it + 1) % (512 / TH) == 0 || it + 1 == job.nit)
+            for (int q = 0; q < 9; ++q)
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+                    float *ia = iacc + (18 * p + q) * TH + tid;
+                    itot[(9 * p + q) * TH + tid] += wide(ia, 9 * TH);
+                    ia[0] = ia[9 * TH] = 0.0f;
+                }
     }
-    float2 *out = static_cast<float2 *>(a.pi) + job.islot(a);
+    double *out = static_cast<double *>(a.pi) + job.islot(a);
 #pragma unroll
     for (int q = 0; q < 9; ++q)
-        *reinterpret_cast<float4 *>(&out[q * a.ns + i]) =
-            make_float4(iacc[q * TH + tid], iacc[(9 + q) * TH + tid], iacc[(18 + q) * TH + tid],
-                        iacc[(27 + q) * TH + tid]);
+        *reinterpret_cast<double2 *>(&out[q * a.ns + i]) = make_double2(itot[q * TH + tid], itot[(9 + q) * TH + tid]);
 }
 
 // ------------------------------------------------------------------ FP64
@@ -580,11 +593,11 @@ struct FoldFF {
     __device__ __forceinline__ double total() const { return static_cast<double>(h) + static_cast<double>(l); }
 };
 
-// FP64 totals of double words (EX).
+// EX: FP64 sums.
 struct FoldEx {
-    using Part = float2;
+    using Part = double;
     double s = 0.0;
-    __device__ __forceinline__ void add(float2 v) { s += static_cast<double>(v.x) + static_cast<double>(v.y); }
+    __device__ __forceinline__ void add(double v) { s += v; }
     __device__ __forceinline__ double total() const { return s; }
 };
 // out[q][p] (+)= the slots of a batch of offsets.
@@ -602,7 +615,7 @@ __global__ void __launch_bounds__(256) fold_kernel(const typename F::Part *pi, i
 }
 
 constexpr size_t mixed_smem(int kp) { return sizeof(float) * kMixedThreads * (2 * NCF + 18 + 36 * kp); }
-constexpr size_t ex_smem(int w) { return sizeof(float) * 32 * w * (2 * NCX + 18 + 36); }
+constexpr size_t ex_smem(int w) { return sizeof(float) * 32 * w * (2 * NCX + 18 + 36 + 36); }
 
 struct SymKind {
     void (*light)(SymArgs), (*heavy)(SymArgs);  // no mass above 1; any masses
