@@ -121,6 +121,14 @@ __device__ __forceinline__ double sum4(const double *v, int n)
     return (s[0] + s[1]) + (s[2] + s[3]);
 }
 
+// x + y of two double words in FP64: the words meet in exact FP32 sums, which
+// leaves two FP64 additions of the three.
+__device__ __forceinline__ double wide_sum(const ff::FF<float> &x, const ff::FF<float> &y)
+{
+    const ff::FF<float> h = ff::two_sum(x.h, y.h), l = ff::two_sum(x.l, y.l), m = ff::two_sum(h.l, l.h);
+    return to_double(h.h) + (to_double(m.h) + to_double(ff::add(m.l, l.l)));
+}
+
 // Sums of the K active particles (listed in act, at most kmax) over the j of
 // [lo, hi), all predicted to tp, written to part[(k * 9 + q) * pstride].  The
 // slice goes through shared memory in chunks of cap records.  L = T / K2 lanes
@@ -246,14 +254,16 @@ __device__ __forceinline__ void eval_slice(const Record &record, double eps2, in
     }
     // mixed: lanes joined by shuffles, in groups of a power of two of them
     const int span = min(32, L & -L);
-    // this thread's sums: doubles, or (hi, lo) words in the FP32 precisions
-    // (EX: the two halves of the packed sums joined by a double-word sum, and
-    // FP64 only where more than 32 iterations went to acc)
+    // this thread's sums: doubles, or (hi, lo) words in the mixed precision
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-        if (PR == 0) {
+        if (PR != 1) {
+            if (PR == 2) {
+                const double s = wide_sum(ff::FF<float>{px[q].h.x, px[q].l.x}, ff::FF<float>{px[q].h.y, px[q].l.y});
+                acc[q] = spilled ? acc[q] + s : s;  // acc is zero in short slices
+            }
             red[tid * 9 + q] = acc[q];
-        } else if (PR == 1) {
+        } else {
             two_sum_acc(ah[q], al[q], __fadd_rn(pm[q].x, pm[q].y));
             for (int o = span >> 1; o > 0; o >>= 1) {
                 const float oh = __shfl_xor_sync(0xffffffffu, ah[q], o);
@@ -262,10 +272,6 @@ __device__ __forceinline__ void eval_slice(const Record &record, double eps2, in
                 al[q] = __fadd_rn(al[q], ol);
             }
             reinterpret_cast<float2 *>(red)[tid * 9 + q] = make_float2(ah[q], al[q]);
-        } else {
-            const ff::FF<float> x = {px[q].h.x, px[q].l.x}, y = {px[q].h.y, px[q].l.y};
-            const ff::FF<float> s = ff::add_accurate(x, y);
-            reinterpret_cast<float2 *>(red)[tid * 9 + q] = make_float2(s.h, s.l);
         }
     }
     __syncthreads();
@@ -282,7 +288,7 @@ __device__ __forceinline__ void eval_slice(const Record &record, double eps2, in
             for (int c = 0; c < 4; ++c)
                 if (e + c * S < nl) {
                     const int at = (k * L + (e + c * S) * stepl) * 9 + q;
-                    if (PR == 0) {
+                    if (PR != 1) {
                         s[c] += red[at];
                     } else {
                         const float2 w = reinterpret_cast<const float2 *>(red)[at];
@@ -301,21 +307,6 @@ __device__ __forceinline__ void eval_slice(const Record &record, double eps2, in
         __syncthreads();
         if (tid < nv)
             part[static_cast<size_t>(tid) * pstride] = sum4(red + tid * S, S);
-    }
-    if (PR == 2 && __syncthreads_or(spilled)) {
-        // long slices: the FP64 sums of the first iterations, added behind
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < 9; ++q)
-            red[tid * 9 + q] = acc[q];
-        __syncthreads();
-        for (int u = tid; u < 9 * K; u += T) {
-            const int k = u / 9, q = u - 9 * k;
-            double s = part[static_cast<size_t>(u) * pstride];
-            for (int e = 0; e < L; ++e)
-                s += red[(k * L + e) * 9 + q];
-            part[static_cast<size_t>(u) * pstride] = s;
-        }
     }
     __syncthreads();
 }

@@ -50,3 +50,22 @@ def test_pair_totals(n, a):
         g.close()
     others = np.setdiff1d(np.arange(0, n, max(1, n // 400)), [a, b]).astype(np.int32)
     check([q[others] for q in sums[1]], [q[others] for q in sums[0]], O.evaluate(mb, x, v, acc, 1e-2, others))
+
+
+# the resident stepper: A and B are the two halves of one lane's packed sums
+@pytest.mark.parametrize("seed", range(8))
+def test_stepper_lanes(seed):
+    nb = nb_gpu()
+    n, h = 4, 2.0 ** -7
+    x, v, acc = (ni.random_state(n, 3 * seed + q + 100) for q in range(3))
+    m0, m1, mb = masses(n, 2, 3)
+    sums = []
+    for m in (m0, m1):
+        g = nb.NBody(m, x, v, 1e-2, precision=3, start_forces=False, dt_max=h)
+        g.set_state({"a": acc, "dt": np.full(n, h)})
+        assert g.run_until(h)[0] == 1
+        st = g.state()
+        sums.append([st[k][:2] for k in "ajs"])
+        g.close()
+    xp, vp = x + h * (v + h / 2 * acc), v + h * acc
+    check(sums[1], sums[0], O.evaluate(mb, xp, vp, acc, 1e-2, np.arange(2, dtype=np.int32)))
