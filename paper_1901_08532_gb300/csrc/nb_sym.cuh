@@ -70,7 +70,11 @@ struct Fold64 {
         e += (s - (t - b)) + (v - b);
         s = t;
     }
-    __device__ __forceinline__ double total() const { return s + e; }
+    __device__ __forceinline__ double total() const
+    {
+        const double r = s + e;
+        return isnan(r) ? s : r;  // an infinite sum leaves no error term
+    }
 };
 
 template <class F, int U>
