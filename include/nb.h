@@ -323,11 +323,15 @@ nb_status nb_get_active(nb_ctx *ctx, int32_t *idx, int64_t cap, int64_t *n_act);
  * injection is one-shot. */
 nb_status nb_inject_fault(nb_ctx *ctx, int32_t kind);
 
-/* Replace the evaluation launch shape (zero fields = automatic). */
+/* Replace the evaluation launch shape (zero fields = automatic).  A shape with
+ * any field set governs every evaluation of the context that runs the
+ * evaluation kernels, also of all particles: the evaluation by unordered
+ * pairs, which the automatic setting takes for complete and large active sets
+ * where it is faster, is then not used. */
 nb_status nb_set_tiles(nb_ctx *ctx, const nb_tiles *tiles);
 
-/* The launch shape the library would use for n_act active particles under
- * the current setting (automatic fields resolved). */
+/* The launch shape of the evaluation kernels for n_act active particles
+ * under the current setting (automatic fields resolved), where they run. */
 nb_status nb_resolve_tiles(nb_ctx *ctx, int64_t n_act, nb_tiles *out);
 
 /* Counters since nb_init: kernels launched by this context and pair

@@ -5,8 +5,9 @@ shapes (i-particles per thread, threads per block, j-tile length, j per
 inner iteration, and for the mixed kernel the lanes per i-particle, 0 being
 the library's own choice; split-j is resolved by the library for each
 shape) through the C-ABI (nb_set_tiles + nb_evaluate, CUDA events on the
-context's stream) and keeps the fastest.  Results are cached per
-(precision, n, n_act bucket) in memory and, optionally, in a JSON file.
+context's stream) and keeps the fastest, or the library's automatic setting
+where no shape beats it.  Results are cached per
+(precision, n, n_act bucket; 0 for all particles) in memory and, optionally, in a JSON file.
 
 Ensembles: tune_ensemble() times candidate cluster shapes (blocks per
 system, threads, j-tile) on fresh copies of an ensemble and keeps the one
@@ -50,8 +51,8 @@ def candidates(precision: int):
 
 
 def time_shape(ctx, shape, active, reps=3):
-    """Mean seconds of one evaluation of `active` (a CUDA int32 tensor) with
-    the given launch shape; None if the library rejects the shape."""
+    """Mean seconds of one evaluation of `active` (a CUDA int32 tensor; None:
+    all particles) with the given launch shape; None if the library rejects the shape."""
     import torch
     import paper_1901_08532_gb300 as nb
     try:
@@ -72,8 +73,15 @@ def time_shape(ctx, shape, active, reps=3):
 
 def tune(ctx, active, reps=3, log=None, cache_file=None):
     """Pick the fastest shape for evaluating `active` on `ctx` and leave it
-    set on the context.  Returns (shape, seconds)."""
-    key = (ctx.precision, ctx.n, _bucket(int(active.numel())))
+    set on the context.  Returns (shape, seconds); the shape {} is the
+    automatic setting, which a list of all particles is timed with as
+    evaluate(None), by unordered pairs where the library takes them.
+
+    A shape governs every evaluation of the context and turns the unordered
+    pairs off, also where all or most particles are active: ctx.set_tiles()
+    goes back to the automatic setting for such steps."""
+    n_act = int(active.numel())
+    key = (ctx.precision, ctx.n, 0 if n_act == ctx.n else _bucket(n_act))
     if key not in _cache and cache_file and os.path.exists(cache_file):
         with open(cache_file) as f:
             for k, v in json.load(f).items():
@@ -82,12 +90,13 @@ def tune(ctx, active, reps=3, log=None, cache_file=None):
         shape, sec = _cache[key]
         ctx.set_tiles(**shape)
         return shape, sec
+    if n_act == ctx.n:
+        active = None
     best = (None, float("inf"))
-    for shape in candidates(ctx.precision):
+    for shape in itertools.chain([{}], candidates(ctx.precision)):
         sec = time_shape(ctx, shape, active, reps)
         if log is not None:
-            log({"shape": shape, "resolved": ctx.resolve_tiles(int(active.numel())) if sec else None,
-                 "seconds": sec})
+            log({"shape": shape, "resolved": ctx.resolve_tiles(n_act) if sec else None, "seconds": sec})
         if sec is not None and sec < best[1]:
             best = (shape, sec)
     if best[0] is None:
