@@ -24,7 +24,10 @@
  *     device memory of the context's device.
  *   - The context owns all of its device memory (allocated in nb_init, the
  *     scratch for partial sums and samples by the first call that needs it,
- *     never under stream capture; released in nb_free) and runs all work on the stream given in
+ *     never under stream capture; released in nb_free).  The scratch of complete
+ *     active sets taken by unordered pairs is at most 256 MB up to 148000
+ *     particles, then at most 1 GB or 144 bytes a particle; where it cannot be
+ *     had, the evaluation kernels need none.  All work runs on the stream in
  *     nb_config.stream (a cudaStream_t; NULL = the legacy default stream).
  *     Entry points that return host data synchronise that stream.
  *   - Softened gravity with G = 1: pair term from particle j on particle i

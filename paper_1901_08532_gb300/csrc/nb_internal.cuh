@@ -53,9 +53,11 @@ struct SymPlan {
 };
 // Bytes of partial sums that a plan may use where it needs more than the two
 // slots (72 B per particle each) of the smallest one: 24 slots, at least
-// 512 MB, at most 1 GB (65536 particles mixed 4.83 ms, with 256 MB 5.05 ms; 2 GB
-// would gain 1 % from 131072 particles).
-constexpr double kSymSlotBytes = 1e9, kSymMinBytes = 512e6, kSymSlots = 24.0;
+// 256 MB, at most 1 GB.  Every context holds them, so a program with many middle-
+// sized ones pays for them many times: at least 512 MB made mixed sums of 65536
+// to 150000 particles 0-5 % faster (65536 4.84 ms with 418 MB, 5.06 with 209 MB) and
+// those of 262144 3 % slower; 2 GB at most would gain 1 % from 131072 particles on.
+constexpr double kSymSlotBytes = 1e9, kSymMinBytes = 256e6, kSymSlots = 24.0;
 
 struct nb_ctx {
     int dev = 0;
