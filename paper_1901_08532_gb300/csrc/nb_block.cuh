@@ -121,12 +121,35 @@ __device__ __forceinline__ double sum4(const double *v, int n)
     return (s[0] + s[1]) + (s[2] + s[3]);
 }
 
-// x + y of two double words in FP64: the words meet in exact FP32 sums, which
-// leaves two FP64 additions of the three.
-__device__ __forceinline__ double wide_sum(const ff::FF<float> &x, const ff::FF<float> &y)
+// s[q] (+)= the halves of the packed double words p[q], joined in FP64: the words
+// meet in exact FP32 sums, which leaves two FP64 additions of the three, and one
+// test covers the conversions.
+__device__ __forceinline__ void join_halves(const ff::FF<float2> (&p)[9], bool add, double (&s)[9])
 {
-    const ff::FF<float> h = ff::two_sum(x.h, y.h), l = ff::two_sum(x.l, y.l), m = ff::two_sum(h.l, l.h);
-    return to_double(h.h) + (to_double(m.h) + to_double(ff::add(m.l, l.l)));
+    float w[9][3];
+    bool normal = true;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        const ff::FF<float> h = ff::two_sum(p[q].h.x, p[q].h.y), l = ff::two_sum(p[q].l.x, p[q].l.y);
+        const ff::FF<float> m = ff::two_sum(h.l, l.h);
+        w[q][0] = h.h;
+        w[q][1] = m.h;
+        w[q][2] = ff::add(m.l, l.l);
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            normal = normal && zero_or_normal(w[q][k]);
+    }
+    auto join = [&](auto wide) {
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const double v = wide(w[q][0]) + (wide(w[q][1]) + wide(w[q][2]));
+            s[q] = add ? s[q] + v : v;
+        }
+    };
+    if (normal)
+        join([](float x) { return to_double_normal(x); });
+    else
+        join([](float x) { return static_cast<double>(x); });
 }
 
 // Sums of the K active particles (listed in act, at most kmax) over the j of
@@ -255,13 +278,11 @@ __device__ __forceinline__ void eval_slice(const Record &record, double eps2, in
     // mixed: lanes joined by shuffles, in groups of a power of two of them
     const int span = min(32, L & -L);
     // this thread's sums: doubles, or (hi, lo) words in the mixed precision
+    if (PR == 2)
+        join_halves(px, spilled, acc);  // acc is zero in short slices
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
         if (PR != 1) {
-            if (PR == 2) {
-                const double s = wide_sum(ff::FF<float>{px[q].h.x, px[q].l.x}, ff::FF<float>{px[q].h.y, px[q].l.y});
-                acc[q] = spilled ? acc[q] + s : s;  // acc is zero in short slices
-            }
             red[tid * 9 + q] = acc[q];
         } else {
             two_sum_acc(ah[q], al[q], __fadd_rn(pm[q].x, pm[q].y));

@@ -169,14 +169,25 @@ __device__ __forceinline__ float to_float(double x)
     return __uint_as_float((hi & 0x80000000u) | (kept + up));
 }
 
+// x as a double (exact), x zero or normal.
+__device__ __forceinline__ bool zero_or_normal(float x)
+{
+    const unsigned m = __float_as_uint(x) & 0x7fffffffu;
+    return m == 0 || (m >> 23) - 1u <= 253u;
+}
+__device__ __forceinline__ double to_double_normal(float x)
+{
+    const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+    return __hiloint2double(static_cast<int>((u & 0x80000000u) | (m == 0 ? 0u : (m >> 3) + (896u << 20))),
+                            static_cast<int>(u << 29));
+}
+
 // x as a double (exact).
 __device__ __forceinline__ double to_double(float x)
 {
-    const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
-    if (m != 0 && (m >> 23) - 1u > 253u)
+    if (!zero_or_normal(x))
         return static_cast<double>(x);  // subnormal, infinite, NaN
-    return __hiloint2double(static_cast<int>((u & 0x80000000u) | (m == 0 ? 0u : (m >> 3) + (896u << 20))),
-                            static_cast<int>(u << 29));
+    return to_double_normal(x);
 }
 
 // ------------------------------------------------------- step quantisation
