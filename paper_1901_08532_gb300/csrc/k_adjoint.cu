@@ -84,7 +84,8 @@ __device__ __forceinline__ void bracket_from_phi(const double (&r)[3], const dou
 // coefficients, so the second pair's gradient with respect to x_k equals the
 // first pair's form evaluated at (r, v, a) with l's cotangents; by linearity
 // both roles need one bracket with g* = m_k g_l - m_l g_k, times q^3.  The mass
-// gradient of m_k is -q^3 Phi(g_l).  For l = k, g* = 0 and Phi = 0 exactly.
+// gradient of m_k is -q^3 Phi(g_l).  For l = k, g* and Phi are zero; the rounding of
+// m_k g_k that the fused g* leaves must not meet q^3 = eps^-3.
 __global__ void __launch_bounds__(kAdjThreads) adjoint_kernel(int n, int lanes, const double *__restrict__ m,
                                                               const double *__restrict__ x,
                                                               const double *__restrict__ v,
@@ -139,7 +140,7 @@ __global__ void __launch_bounds__(kAdjThreads) adjoint_kernel(int n, int lanes, 
             }
             const double R = fma(r[0], r[0], fma(r[1], r[1], fma(r[2], r[2], eps2)));
             const double q = nbk::rsqrt_fp64(R);
-            const double q2 = q * q, q3 = q * q2;
+            const double q2 = q * q, q3 = l0 + e == k ? 0.0 : q * q2;
             const double al = fma(r[0], vr[0], fma(r[1], vr[1], r[2] * vr[2])) * q2;
             const double be = fma(fma(vr[0], vr[0], fma(vr[1], vr[1], vr[2] * vr[2])) +
                                       fma(r[0], ar[0], fma(r[1], ar[1], r[2] * ar[2])),
