@@ -651,7 +651,7 @@ void nb_sym_plan_shape(const SymShape &kd, int kind, int64_t n, int sms, SymPlan
     const int64_t T = (n + kd.tile - 1) / kd.tile, D = T / 2 + 1;
     const double slot = static_cast<double>(kd.bytes) * static_cast<double>(T * kd.tile);
     const double budget = std::min(kSymSlotBytes, std::max(kSymMinBytes, kSymSlots * slot));
-    const int64_t slots = max_bytes ? static_cast<int64_t>(std::min(budget, static_cast<double>(max_bytes)) / slot)
+    const int64_t slots = max_bytes ? static_cast<int64_t>(static_cast<double>(max_bytes) / slot)
                                     : std::max<int64_t>(2, static_cast<int64_t>(budget / slot));
     const int subs = kd.tile / kd.threads;
     for (const int k : {1, 2, 4, 8})

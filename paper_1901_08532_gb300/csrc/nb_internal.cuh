@@ -292,7 +292,7 @@ nb_tiles nb_auto_tiles(const nb_ctx *c, int64_t n_act, const nb_tiles &req, int6
                        double *us = nullptr);
 cudaError_t nb_eval_smem_setup();
 // k_sym.cu
-// max_bytes: of partial sums (0: as many as a context's own plan may use)
+// max_bytes: of partial sums that there are (0: as many as a context's own plan may use)
 SymPlan nb_sym_plan(int precision, int64_t n, int sms, size_t max_bytes = 0);
 cudaError_t nb_sym_smem_setup();
 // jb, np: predicted particles and row stride; light: no mass is above 1 (FP64: of
