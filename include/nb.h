@@ -182,7 +182,10 @@ nb_status nb_get_predicted(nb_ctx *ctx, double *xp, double *vp, double *ap);
  * [n_act][3] doubles; they are host pointers, or device pointers when
  * out_on_device != 0; any of them may be NULL (results are then only kept
  * for nb_correct).  Indices are checked on the host when active is a host
- * pointer; device lists are trusted.
+ * pointer; device lists are trusted and not looked at.  All particles, as NULL
+ * or in order in a host list, are taken by unordered pairs where that is
+ * faster, which adds in another order than a device list of the same particles:
+ * the results agree to the rounding of the precision.
  * Errors: NB_EINVAL (n_act < 0 or > n, bad index), NB_ESTATE (no prediction yet). */
 nb_status nb_evaluate(nb_ctx *ctx, const int32_t *active, int64_t n_act,
                       int active_on_device, double *acc, double *jerk,
@@ -253,8 +256,10 @@ nb_status nb_correct(nb_ctx *ctx, double t);
  * section 3, opening paragraph: the predictor, evaluation and corrector
  * stages, in that order), entirely on the device: t_next = min_i(t_i + dt_i),
  * the active set {i : t_i + dt_i == t_next} (ascending indices), predict all,
- * evaluate the active set, correct it.  *t_out and *n_act_out (either may
- * be NULL) receive the step's time and active count. */
+ * evaluate the active set, correct it.  A large set is taken in two parts where
+ * that is faster (its members among themselves by unordered pairs), which adds
+ * in another order than nb_evaluate of the same list.  *t_out and *n_act_out
+ * (either may be NULL) receive the step's time and active count. */
 nb_status nb_step(nb_ctx *ctx, double *t_out, int64_t *n_act_out);
 
 /* Block steps (section 2; the stages of section 3, and the time-step
@@ -302,7 +307,9 @@ nb_status nb_angmom(nb_ctx *ctx, double L[3], double *labs);
  * every shared step; here the state stays in device memory and this call
  * copies it out on request.
  * nb_get_state followed by nb_set_state on a fresh context (start_forces =
- * 0) resumes an integration bit for bit. */
+ * 0) of the same settings resumes an integration bit for bit, as long as both
+ * contexts can allocate their scratch (see the conventions above): without it
+ * the sums are added in another order. */
 nb_status nb_get_state(nb_ctx *ctx, double *x, double *v, double *a, double *j,
                        double *s, double *c, double *t, double *dt);
 

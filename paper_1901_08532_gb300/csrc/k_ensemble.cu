@@ -1049,7 +1049,7 @@ cudaError_t max_clusters_kind(nb_ensemble *e, int *out)
 // 16 blocks (ms): FP64 32 systems of 256-2048 30.5 / 28.1 / 14.7 (8 before),
 // 100 of 256-1024 15.8 / 9.2 / 11.8, 256 of 256-16384 - / 60.9 / 66.6 s; mixed
 // 32 of 256-4096 6.9 / 4.8 / 3.8 (4 before), 128 10.1 / 6.2 / 10.5, 256 of
-// 256-16384 2.43 / 1.28 / 1.65 s; EX 100 of 256-1500 8.8 / 4.8 / 6.0 (16 before),
+// 256-16384 2.43 / 1.28 / 1.65 s; EX 100 of 256-1500 7.3-8.8 / 4.9 / 6.1 (16 before),
 // 256 of 256-16384 - / 11.3 / 11.1 s.  The estimate takes the best one in each.
 int default_ctas(nb_ensemble *e)
 {

@@ -25,12 +25,13 @@
 // and corrector by component, sums over lanes and over blocks by value, each
 // output a short chain of one thread), and comparisons use integers.  Time
 // per step with about 13 active particles, before -> after: FP64 N = 1024
-// 39.2 -> 18.1 us, EX N = 8192 46.1 -> 20.7 us, mixed N = 65536 58.0 -> 31.6 us.
+// 39.2 -> 18.1 us, EX N = 8192 46.1 -> 21.3 us, mixed N = 65536 58.0 -> 31.6 us.
 // It returns to the host when the next active set holds more than
 // kStepSmall particles, which it leaves listed (the host then runs that step
-// with the tuned evaluation kernels and needs no scheduler pass, about 28 us), when the next block time passes t_end, or after an
-// error flag.  Every block takes the same branch at every barrier (decisions
-// come from the same global values), and no block waits on a flag.
+// with the tuned evaluation kernels and needs no scheduler pass, about 28 us),
+// when the next block time passes t_end, or after an error flag.  Every block
+// takes the same branch at every barrier (decisions come from the same global
+// values), and no block waits on a flag.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -53,7 +54,8 @@ constexpr int kStepSmall = 128;  // active sets up to this size are stepped on t
 // which a block has 256 threads instead of 128: more warps predict a long
 // slice, fewer make every sum over lanes and blocks shorter (us a step, 128 / 256
 // threads: EX N = 8192 20.7 / 21.6, EX 20000 30.8 / 26.8, mixed 65536
-// 38.5 / 31.6; FP64 N = 1024 with 8 and 16 particles per block 18.1 and 19.4).
+// 38.5 / 31.6; FP64 N = 1024 with 8 and 16 particles per block 18.1 and 19.4; the
+// EX figures without the lanes' FP64 join, 0.6 us).
 constexpr int kSliceFp64 = 8, kSliceFp32 = 16, kSliceWide = 96;
 constexpr int kChunkCap = 1024;  // j-records per shared-memory chunk
 

@@ -66,8 +66,8 @@ __host__ __device__ constexpr int mixed_tile(int kp) { return kMixedThreads * 2 
 // no mass is above 1 (LIGHT), m q^3 is no larger than it and leaves the range with it or
 // before, so it may be formed once for both.  Larger masses, such as G m in metres
 // or centimetres, come in before the second power of q, as in the ordinary
-// kernels: one product more, 3.6 % (mixed) and 1.5 % (EX) of the time (524288
-// particles mixed 296 / 306 ms, 40000 EX 15.0 / 15.2 ms).
+// kernels: one product more, 3.6 % (mixed) and 1.6 % (EX) of the time (524288
+// particles mixed 296 / 307 ms, 16384 EX 2.54 / 2.58 ms).
 template <bool LIGHT>
 __device__ __forceinline__ void mass_factors(float2 q, float2 q2, float2 mj, float2 nmi, float2 &mu, float2 &nu)
 {
@@ -155,9 +155,9 @@ __device__ __forceinline__ void load_tile_mixed(const SymArgs &a, float *dst, in
 // ordinary kernel's at 16384 to 65536 particles.
 //
 // All particles, prediction not included, ordinary kernel -> this one:
-// 4096 51 -> 39 us, 8192 150 -> 111, 20011 744 -> 500, 65536 7.26 -> 4.80 ms,
-// 131072 28.6 -> 18.7 ms, 2^20 1.813 -> 1.178 s.  Below about 3500 particles the ordinary kernels
-// are faster (3000: 34 us against 39).
+// 4096 51 -> 39 us, 8192 150 -> 111, 20011 744 -> 500, 65536 7.26 -> 5.05 ms,
+// 131072 28.6 -> 19.2 ms, 2^20 1.813 -> 1.178 s.  Below about 3500 particles the
+// ordinary kernels are faster (3000: 34 us against 39).
 template <int KP, bool LIGHT>
 __global__ void __launch_bounds__(kMixedThreads, 2) sym_mixed_kernel(SymArgs a)
 {

@@ -480,8 +480,8 @@ nb_status nb_init(nb_ctx **out, int64_t n, const double *m, const double *x, con
         g_init_err = msg;
         return NB_EINVAL;
     }
-    // eps^2 must be an FP32 normal number (FP64 rsqrt estimate); the mixed
-    // path also needs m / eps^3 to stay below the FP32 range.
+    // FP32 pair arithmetic needs eps^2 and m / eps^3 within the FP32 range; the
+    // bound of FP64 lies far inside its own.
     const bool fp32_range = nb_jrows(cf.precision) > 0;
     const double eps_min = fp32_range ? std::ldexp(1.0, -40) : std::ldexp(1.0, -60);
     if (!(eps >= eps_min) || !(eps <= 1e18)) {

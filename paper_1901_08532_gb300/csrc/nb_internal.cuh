@@ -213,7 +213,8 @@ constexpr unsigned long long kWaitLimitNs = 1000000000ull;  // 1 s
 // third-order step).  x = m 4^k with m in [1, 4); y = the FP32 hardware estimate
 // of 1/sqrt(m); its residual r = 1 - m y^2 in FP32 (y^2 exactly as a pair, m as
 // a pair) gives the correction y r / 2, added to y's bits as an integer and
-// rounded to 26 bits: y0, within 2^-26.  Then y0^2 is exact, h = 1 - x y0^2
+// rounded to 26 bits: y0, within 2^-26.  Then y0^2 is exact (also where it is
+// subnormal, x > 2^1022: y0 is a multiple of 2^-26 2^-k there), h = 1 - x y0^2
 // rounds once, and y = y0 + (y0 / 2)(1 + 3 h / 4) h, the series of
 // (1 - h)^(-1/2) to h^2 (what is left is below 2^-75), rounds once more: the
 // factor 1 + 3 h / 4 goes into the bits of y0 / 2 as an integer too.
