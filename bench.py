@@ -70,7 +70,7 @@ def set_device_peaks(torch, dev):
 # one ncu pass each); valid only for the kernel source it was measured on (the
 # sha256 prefix of TRAFFIC_FILES under csrc).
 TRAFFIC_FILES = ("k_sym.cu", "nb_sym.cuh", "nb_device.cuh")
-TRAFFIC = {"kernel_sha": "24b465cc08bc62a9", "bytes_per_evaluation": 155851.976704e6 + 103905.487872e6,
+TRAFFIC = {"kernel_sha": "884ebbb0d4528a43", "bytes_per_evaluation": 156095.416320e6 + 103928.877312e6,
            "source": "ncu dram__bytes_read.sum + dram__bytes_write.sum over the evaluation's launches"}
 # FP32-pipe operations per unordered pair in sym_mixed_kernel; per interaction half of them.
 SYM_OPS_PER_PAIR = 63

@@ -208,9 +208,9 @@ nb_status eval_on_device(nb_ctx *c, const int32_t *act_dev, int64_t n_act, bool 
 // 15 % apart and the step slower by a tenth), and where 0.4 of that share is below
 // 15 us the ordinary form is taken without a plan (planning costs the host 4 us).
 // Whole steps, ordinary -> in two parts: 65536 particles EX with 0.25 / 0.5 / 0.95 of
-// them active 15.3 / 31.1 / 59.8 -> 14.1 / 25.7 / 39.2 ms, mixed 1.93 / 3.73 / 6.88 -> 1.82 /
-// 3.18 / 4.92 ms; 8192 FP64 1.58 / 3.10 / 6.00 -> 1.47 / 2.53 / 3.87 ms; 16384 mixed, 0.7,
-// 403 -> 357 us.
+// them active 15.3 / 31.1 / 59.8 -> 14.1 / 25.5 / 39.2 ms, mixed with 0.5 / 0.95 3.73 / 6.88 ->
+// 3.18 / 5.13 ms; 8192 FP64 3.10 / 6.00 -> 2.54 / 3.87 ms (0.25 of either stays in the
+// ordinary form).
 struct FrontPlan {
     int64_t front = 0;
     SymPlan pairs;
